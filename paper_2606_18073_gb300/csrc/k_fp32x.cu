@@ -400,37 +400,16 @@ __global__ void __launch_bounds__(kThreads) kx_apply_column(Dims D, DevA<float, 
     }
 }
 
-__global__ void kx_dense_sketch_pair(Dims D, BulkX B, Small S, const double* __restrict__ SA,
-                                     const double* __restrict__ SL) {
-    if (S.sc->stop) return;
-    const int d = S.sc->d;
-    if (d >= D.dmax) return;
-    const int row = blockIdx.x * kWarps + warp_id();
-    const bool isA = row < D.s;
-    const int r = isA ? row : row - D.s;
-    if (r >= D.s) return;
-    double a = 0.0;
-    if (isA) {
-        const float2* u = B.AW + (size_t)d * D.m;
-        for (int64_t j = lane_id(); j < D.m; j += 32) a += SA[(size_t)r * D.m + j] * dval(u[j]);
-    } else {
-        for (int64_t j = lane_id(); j < D.p; j += 32) a += SL[(size_t)r * D.p + j] * B.tmp_p[j];
-    }
-    a = warp_sum(a);
-    if (lane_id() == 0) (isA ? S.partA : S.partL)[r] = a;
-}
-
 static int x_apply_blocks(const Dims& D);
 
 cudaError_t launchx_gaussian_sketch(const Dims& D, const DevA<float, float>& A, const DevL& L, const BulkX& B,
-                                    const Small& S, const double* SA, const double* SL, cudaStream_t st) {
+                                    const Small& S, const double* SA, const double* SL, const DenseWork& K,
+                                    cudaStream_t st) {
     if (A.kind == SGKS_OP_CONV2D) { carveout_once((const void*)kx_apply_column<false>); kx_apply_column<false><<<x_apply_blocks(D), kThreads, 0, st>>>(D, A, L, B, S); }
     else { carveout_once((const void*)kx_apply_column<true>); kx_apply_column<true><<<x_apply_blocks(D), kThreads, 0, st>>>(D, A, L, B, S); }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    carveout_once((const void*)kx_dense_sketch_pair);
-    kx_dense_sketch_pair<<<(2 * D.s + kWarps - 1) / kWarps, kThreads, 0, st>>>(D, B, S, SA, SL);
-    return cudaGetLastError();
+    return launch_dense_pair<float2, double>(D, B.AW, B.tmp_p, S, SA, SL, K, st);
 }
 
 __global__ void kx_to_float(const float2* __restrict__ in, float* out, int64_t n) {

@@ -14,7 +14,7 @@
 //   is bit-reproducible and no floating-point atomics are used.  (A fused scatter into shared
 //   memory accumulators was measured first: resolving lane collisions with __match_any_sync
 //   made it latency-bound at ~34 us per column for the 256^2 deblurring problem.)
-// k_dense_sketch_pair: S_A u and S_L t for the Gaussian sketch, one warp per sketch row.
+// Dense sketches (Gaussian, SRTT): k_dense.cu.
 #include "sgks_internal.cuh"
 
 namespace sgks {
@@ -138,37 +138,6 @@ __global__ void __launch_bounds__(kThreads) k_sketch_gather_vec(const int32_t* _
     if (threadIdx.x == 0) out[r] = t;
 }
 
-template <typename T, typename V>
-__global__ void k_dense_sketch_pair(Dims D, Bulk<T> B, Small S, const double* __restrict__ SA,
-                                    const double* __restrict__ SL) {
-    if (S.sc->stop) return;
-    const int d = S.sc->d;
-    if (d >= D.dmax) return;
-    const int row = blockIdx.x * kWarps + warp_id();
-    const bool isA = row < D.s;
-    const int r = isA ? row : row - D.s;
-    if (r >= D.s) return;
-    const T* v = isA ? B.AW + (size_t)d * D.m : B.tmp_p;
-    const int64_t len = isA ? D.m : D.p;
-    const double* SG = isA ? SA : SL;
-    double a = 0.0;
-    for (int64_t j = lane_id(); j < len; j += 32) a += SG[(size_t)r * len + j] * (double)v[j];
-    a = warp_sum(a);
-    if (lane_id() == 0) (isA ? S.partA : S.partL)[r] = a;
-}
-
-// Dense (Gaussian) sketch of a plain vector: part[i] = sum_j SG[i*len + j] v[j].
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_dense_sketch(const double* __restrict__ SG, const T* __restrict__ v,
-                                                           int64_t len, int s, double* part) {
-    const int row = blockIdx.x * kWarps + warp_id();
-    if (row >= s) return;
-    double a = 0.0;
-    for (int64_t j = lane_id(); j < len; j += 32) a += SG[(size_t)row * len + j] * (double)v[j];
-    a = warp_sum(a);
-    if (lane_id() == 0) part[row] = a;
-}
-
 // --------------------------------------------------------------------------- launchers
 static int apply_blocks(const Dims& D, bool warpa = false) {
     const int64_t slabs = (D.m + 31) / 32 + (D.p + 31) / 32;
@@ -234,22 +203,13 @@ cudaError_t launch_sketch_vec(const int32_t* ptr, const uint32_t* idx, const voi
     return cudaGetLastError();
 }
 
-cudaError_t launch_dense_sketch(const double* SG, const void* v, int vdt, int64_t len, int s, double* part,
-                                cudaStream_t st) {
-    if (vdt == SGKS_F32) { carveout_once((const void*)k_dense_sketch<float>); k_dense_sketch<float><<<(s + kWarps - 1) / kWarps, kThreads, 0, st>>>(SG, (const float*)v, len, s, part); }
-    else { carveout_once((const void*)k_dense_sketch<double>); k_dense_sketch<double><<<(s + kWarps - 1) / kWarps, kThreads, 0, st>>>(SG, (const double*)v, len, s, part); }
-    return cudaGetLastError();
-}
-
 template <typename T, typename V>
 cudaError_t launch_gaussian_sketch(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B,
-                                   const Small& S, const double* SA, const double* SL, cudaStream_t st) {
+                                   const Small& S, const double* SA, const double* SL, const DenseWork& K,
+                                   cudaStream_t st) {
     cudaError_t e = launch_apply_column<T, V>(D, A, L, B, S, st);
     if (e != cudaSuccess) return e;
-    const int blocks = (2 * D.s + kWarps - 1) / kWarps;
-    carveout_once((const void*)k_dense_sketch_pair<T, V>);
-    k_dense_sketch_pair<T, V><<<blocks, kThreads, 0, st>>>(D, B, S, SA, SL);
-    return cudaGetLastError();
+    return launch_dense_pair<T, T>(D, B.AW, B.tmp_p, S, SA, SL, K, st);
 }
 
 // out[i] = scale * sum_{b < nb} part[b*len + i], summed in b order.
@@ -376,7 +336,7 @@ cudaError_t launch_apply_new_column(const Dims& D, const DevA<T, V>& A, const De
                                                     cudaStream_t);                                          \
     template cudaError_t launch_gaussian_sketch<T, V>(const Dims&, const DevA<T, V>&, const DevL&,          \
                                                       const Bulk<T>&, const Small&, const double*,          \
-                                                      const double*, cudaStream_t);
+                                                      const double*, const DenseWork&, cudaStream_t);
 SGKS_INST_SK(float, float)
 SGKS_INST_SK(double, float)
 SGKS_INST_SK(double, double)

@@ -119,6 +119,7 @@ struct Engine : EngineBase {
     cudaStream_t st = nullptr;
     const double* gSA = nullptr;
     const double* gSL = nullptr;
+    DenseWork DW{};                 // of the dense sketches
     double* part_setup = nullptr;   // [nbS][8]
     int nbS = 1;
     int* d_err = nullptr;
@@ -157,7 +158,7 @@ struct Engine : EngineBase {
         if (e != cudaSuccess) return e;
         // S_A b
         const int tdt = sizeof(T) == 4 ? SGKS_F32 : SGKS_F64;
-        if (gSA) e = launch_dense_sketch(gSA, B.b, tdt, D.m, D.s, S.partA, st);
+        if (gSA) e = launch_dense_sketch(gSA, B.b, tdt, D.m, D.s, DW, S.partA, st);
         else e = launch_sketch_vec(SK.ptrA, SK.idxA, B.b, tdt, sizeof(T) == 4, D.s, S.partA, st);
         if (e == cudaSuccess) e = launch_reduce_rows(S.partA, 1, D.s, D.sketch_scale, S.Sb, st);
         if (e != cudaSuccess) return e;
@@ -186,7 +187,7 @@ struct Engine : EngineBase {
     }
 
     cudaError_t sketch() {
-        if (gSA) return launch_gaussian_sketch<T, V>(D, A, L, B, S, gSA, gSL, st);
+        if (gSA) return launch_gaussian_sketch<T, V>(D, A, L, B, S, gSA, gSL, DW, st);
         return launch_sketch_column<T, V>(D, A, L, B, S, SK, st);
     }
 
@@ -535,7 +536,7 @@ struct Engine : EngineBase {
         const double* SG = isA ? gSA : gSL;
         double* part = isA ? S.partA : S.partL;
         cudaError_t e;
-        if (SG) e = launch_dense_sketch(SG, in, vdt, isA ? D.m : D.p, D.s, part, st);
+        if (SG) e = launch_dense_sketch(SG, in, vdt, isA ? D.m : D.p, D.s, DW, part, st);
         else e = launch_sketch_vec(isA ? SK.ptrA : SK.ptrL, isA ? SK.idxA : SK.idxL, in, vdt, acc_f32, D.s, part, st);
         if (e != cudaSuccess) return e;
         return launch_reduce_rows(part, 1, D.s, D.sketch_scale, out, st);
@@ -670,7 +671,7 @@ struct EngineX : Engine<float, float> {
     BulkX X{};
 
     cudaError_t sketchx() {
-        if (gSA) return launchx_gaussian_sketch(D, A, L, X, S, gSA, gSL, st);
+        if (gSA) return launchx_gaussian_sketch(D, A, L, X, S, gSA, gSL, DW, st);
         return launchx_sketch_column(D, A, L, X, S, SK, st);
     }
 
@@ -1168,6 +1169,12 @@ static int build_engine(sgks_handle* h, const sgks_op* op, const sgks_reg* reg, 
     AL(S.rre_hist, (size_t)o.max_iters + 1);
     AL(S.sc, 1);
     AL(E->part_setup, (size_t)E->nbS * 8);
+    size_t dense_part = 0, dense_cnt = 0;
+    if (gauss) {
+        dense_work_size(D.m, D.p, s, &dense_part, &dense_cnt);
+        AL(E->DW.part, dense_part);
+        AL(E->DW.cnt, dense_cnt);
+    }
     if (o.flags & SGKS_FLAG_RECORD) AL(E->yhist, (size_t)(o.max_iters + 1) * (o.n_refine + 1) * dm);
     if (EG) {
         if (!D.fast_small) return fail(h, SGKS_ERR_INVALID, "GKS needs the on-chip stacked solve (sketch_rows too large)");
@@ -1191,6 +1198,7 @@ static int build_engine(sgks_handle* h, const sgks_op* op, const sgks_reg* reg, 
     if (e == cudaSuccess && xs) e = cudaMemsetAsync(xs, 0, sizeof(T) * D.n, h->st);
     if (e == cudaSuccess && xform) e = cudaMemsetAsync(EX->X.xs, 0, 8 * D.n, h->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(E->d_err, 0, sizeof(int), h->st);
+    if (e == cudaSuccess && E->DW.cnt) e = cudaMemsetAsync(E->DW.cnt, 0, sizeof(int) * dense_cnt, h->st);
 
     if (e != cudaSuccess) return cuda_fail(h, e, "workspace initialisation");
     {

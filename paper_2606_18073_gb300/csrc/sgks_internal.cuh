@@ -716,6 +716,17 @@ struct SketchCSR {
     const uint32_t* idxL;
 };
 
+// Dense sketches (k_dense.cu): a matrix-vector product in row groups and nc column chunks of C, its
+// partials and the arrival counter of each row group (zero between launches).
+struct DensePlan {
+    int64_t C;
+    int nc, groups;
+};
+struct DenseWork {
+    double* part;
+    int* cnt;
+};
+
 // S_L re-blocked by column chunks of t = L w (batched compensated forms): chunk c covers the
 // columns q in [c C, c C + C); the entries of sketch row r in chunk c are ent[seg[c s + r] ..
 // seg[c s + r + 1]), each (q - c C) | sign << 31, in the row's own order.  nchunks = 0: not built.
@@ -787,11 +798,17 @@ cudaError_t launch_sketch_column(const Dims& D, const DevA<T, V>& A, const DevL&
                                  const Small& S, const SketchCSR& SK, cudaStream_t st);
 template <typename T, typename V>
 cudaError_t launch_gaussian_sketch(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B,
-                                   const Small& S, const double* SA, const double* SL, cudaStream_t st);
+                                   const Small& S, const double* SA, const double* SL, const DenseWork& K,
+                                   cudaStream_t st);
+// part and cnt elements of the DenseWork of an s x m and an s x p sketch
+void dense_work_size(int64_t m, int64_t p, int s, size_t* part, size_t* cnt);
+template <typename TA, typename TL>
+cudaError_t launch_dense_pair(const Dims& D, const TA* AW, const TL* lw, const Small& S, const double* SA, const double* SL,
+                              const DenseWork& K, cudaStream_t st);
 cudaError_t launch_sketch_vec(const int32_t* ptr, const uint32_t* idx, const void* v, int vdt, bool acc_f32, int s,
                               double* out, cudaStream_t st);
-cudaError_t launch_dense_sketch(const double* SG, const void* v, int vdt, int64_t len, int s, double* part,
-                                cudaStream_t st);
+cudaError_t launch_dense_sketch(const double* SG, const void* v, int vdt, int64_t len, int s, const DenseWork& K,
+                                double* out, cudaStream_t st);
 cudaError_t build_sketch_csr(uint64_t key, int64_t h, int s, int zeta, int32_t* ptr, uint32_t* idx, int* err,
                              cudaStream_t st);
 cudaError_t launchx_sketch_gather_col(const Dims& D, const float2* AW, const double* lw, const SketchCSR& SK,
@@ -833,7 +850,8 @@ cudaError_t launchx_gradient(const Dims& D, const DevA<float, float>& A, const D
                              const Small& S, bool refine, cudaStream_t st);
 cudaError_t launchx_to_float(const float2* in, float* out, int64_t n, cudaStream_t st);
 cudaError_t launchx_gaussian_sketch(const Dims& D, const DevA<float, float>& A, const DevL& L, const BulkX& B,
-                                    const Small& S, const double* SA, const double* SL, cudaStream_t st);
+                                    const Small& S, const double* SA, const double* SL, const DenseWork& K,
+                                    cudaStream_t st);
 
 // setup helpers (sgks_setup.cu)
 template <typename T, typename V>
