@@ -77,6 +77,80 @@ struct Dot2 {
     __device__ __forceinline__ double to_double() const { return (double)p + (double)s; }
 };
 
+// Two floats in one 64-bit register pair.  GB300 takes one instruction for both (add, subtract,
+// multiply, fused multiply-add of .f32x2, each lane rounded as the scalar instruction), so a
+// float-float loop issues half as many instructions for the same work of the FP32 pipe.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Two Dot2 accumulators side by side: the operations of Dot2 with the same roundings on both halves.
+struct Dot2x2 {
+    f32x2 p = 0, s = 0;   // (+0, +0)
+    __device__ __forceinline__ void accumulate(f32x2 h, f32x2 r) {   // (h, r): a product or a float-float value
+        const f32x2 t = add2(p, h), bb = sub2(t, p);
+        const f32x2 q = add2(sub2(p, sub2(t, bb)), sub2(h, bb));
+        p = t;
+        s = add2(s, add2(q, r));
+    }
+    // a * b; the error of the product is taken negated, fl(ab) - ab = fma(-a, b, fl(ab)), so that only
+    // the coefficient's sign is flipped (integer units), never a 64-bit operand of the FP32 pipe
+    __device__ __forceinline__ void add_prod(f32x2 a, f32x2 b) {
+        const f32x2 h = mul2(a, b), nr = fma2(a ^ 0x8000000080000000ull, b, h);
+        const f32x2 t = add2(p, h), bb = sub2(t, p);
+        const f32x2 q = add2(sub2(p, sub2(t, bb)), sub2(h, bb));
+        p = t;
+        s = add2(s, sub2(q, nr));
+    }
+    __device__ __forceinline__ void add_prod2(f32x2 a, f32x2 bh, f32x2 bl) {
+        add_prod(a, bh);
+        s = fma2(a, bl, s);
+    }
+    __device__ __forceinline__ void merge(const Dot2x2& o) { accumulate(o.p, o.s); }
+    __device__ __forceinline__ void renorm() { value(p, s); }   // as Dot2::renorm
+    __device__ __forceinline__ void value(f32x2& hi, f32x2& lo) const {   // renormalised float-float pairs
+        const f32x2 t = add2(p, s), bb = sub2(t, p);
+        lo = add2(sub2(p, sub2(t, bb)), sub2(s, bb));
+        hi = t;
+    }
+    __device__ __forceinline__ Dot2 half(int i) const {
+        const float2 a = unpack2(p), b = unpack2(s);
+        Dot2 d;
+        d.p = i ? a.y : a.x;
+        d.s = i ? b.y : b.x;
+        return d;
+    }
+};
+
 // Dot2's error grows with the number of terms in one accumulator: the collected errors are
 // summed in plain FP32 (the bound is u|sum| + gamma_n^2 sum|p_i|, gamma_n ~ n u).  A CPU emulation
 // of these kernels' Dot2 on 229-term dot products with terms of both signs measured the error at

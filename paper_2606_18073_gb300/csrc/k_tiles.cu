@@ -1,302 +1,516 @@
-// Pixel-tiled forward pass of a CSR operator for the batched compensated forms.
+// Pixel-tiled passes of a CSR operator on an image geometry, batched compensated forms: u = A w and
+// r = A^T e + lambda L^T L x.
 //
-// A ray-based operator (CT, travel-time tomography) has rows that are long lines through the
-// image: the CSR pass u_i = A w_i gathers, for every nonzero, the instance vector w[col][0..B) --
-// 512 bytes per nonzero for 64 float-float instances, 30 GB per pass on the 512^2 CT operator,
-// more than the L2 holds once w is float-float.  Here the image is cut into TX x TY pixel tiles:
-// a CTA stages one tile of w (IC instances) in shared memory once, walks the (ray, tile) segments
-// crossing the tile and writes one float-float partial per segment and instance; a second kernel
-// sums each ray's partials in the order of its segments (the order of the row's entries), so the
-// result is the same on every run.  The operator is re-blocked once per batch on the host:
-// segments are the runs of a row's entries that fall in one tile (entries stably sorted by tile),
-// stored tile-major, each entry as (local pixel index, value) in 8 bytes.
-#include <string.h>
-
+// A ray operator (CT, travel-time tomography) has rows that are long lines through the image, so a
+// CSR pass gathers one whole instance vector per nonzero: 512 bytes each for 64 float-float
+// instances, 30 GB per pass on the 512^2 CT operator.  Here the image is cut into pixel tiles and a
+// CTA keeps the gathered side in shared memory:
+//   forward    a tile of w (IC instances); the CTA walks the (ray, tile) segments that cross the tile
+//              and leaves one float-float partial per segment and instance, which kbx_seg_reduce adds
+//              up ray by ray in the order of the row's entries;
+//   transposed the rays that cross a tile are staged in shared memory a few hundred at a time (rays of a
+//              tile in ascending order) and every pixel of the tile adds its entries of the stage to
+//              accumulators that stay in registers; the stencil and lambda finish the row, so the
+//              gradient is written once and e is read once per crossing (ray, tile) pair.
+//
+// What bounds both is the FP32 pipe: 11 operations per entry and instance of Dot2 (ff.cuh) are
+// 42.3 G on the CT batch (60 M entries, 64 instances), 1.05 ms at 40.3 T/s; Dot2 alone, on registers,
+// reaches 33 T/s.  Measured there (float-float): A w 2.82 -> 1.93 ms with kbx_seg_reduce's 0.25, A^T e
+// 3.07 -> 2.00 ms against the row kernel's 512-byte gathers.  A batch of one on a 301^2 image: 105 -> 62
+// and 92 -> 43 us.  Therefore
+// - a lane works on two instances at once with the .f32x2 instructions, 11 per entry, which leaves half
+//   of the issue slots for the loads and addresses; with 16 instances it takes two such pairs, so that
+//   an entry's load (which the lanes of a row repeat) serves twice as many products;
+// - staged values lie as pairs (hi0, hi1, lo0, lo1), so that one 16-byte load gives two operands;
+// - 16 instances per CTA make a staged float-float row 128 bytes, all banks once: the eight lanes of a
+//   load phase read half of one row and the other half of another, without bank conflicts;
+// - entries are stored for groups of four rows (segments, or pixels), interleaved: entries k and
+//   k + 1 of a row side by side (slot, slot, value, value), the four rows next to each other, so a
+//   warp's entry load is one contiguous line.  Segments of a tile are sorted by length, so that the
+//   four of a group run equally long; shorter rows are filled with entries of value 0 on a slot
+//   that holds 0.
+// A batch of one takes the two entries of a pair in the two halves instead of two instances.
+// The layouts are built on the device, once per operator (k_tile_build.cu).
 #include <algorithm>
-#include <numeric>
-#include <string>
-#include <vector>
 
-#include "batch_common.cuh"
-#include "ff.cuh"
+#include "batchx_common.cuh"
 
 namespace sgks {
 
-__device__ __forceinline__ void tacc(Dot2& a, float coef, float w) { a.add_prod(coef, w); }
-__device__ __forceinline__ void tacc(Dot2& a, float coef, float2 w) { a.add_prod2(coef, w.x, w.y); }
+namespace {
 
-template <typename TW>
-__device__ __forceinline__ TW tzero() { return TW{}; }
+// Lane layout for IC staged instances: a lane takes VV of them (VV = 1: IC = 1, the halves of an
+// .f32x2 operand are then the two entries of a pair), G = IC / VV lanes per row.
+template <int IC>
+struct Lanes {
+    static constexpr int VV = IC >= 16 ? 4 : (IC >= 2 ? 2 : 1);
+    static constexpr int NP = VV == 4 ? 2 : 1;   // .f32x2 accumulators of a lane
+    static constexpr int G = IC / VV;
+    // Threads: two such pairs per lane take 80 registers, 256 threads then fill an SM three times over;
+    // with fewer instances a tile's CTA is small work and takes 512.
+    static constexpr int threads = IC >= 16 ? 256 : 512;
+};
 
-// Partials of the segments of one tile for IC instances.  grid: ntiles * (B / IC) CTAs of
-// kThreads threads; thread (ig, sl) takes VV consecutive instances c IC + ig VV + [0, VV) (one
-// 16-byte shared-memory load per entry serves all VV) and segments sl, sl + NSL, ... of the tile.
-// Shared-memory slot of local pixel q (row-major in a tile of width TX, TX even): pixel rows
-// swap neighbouring slots on odd rows.  A 16-byte shared load phase serves the pixels of two
-// neighbouring segments, which on rays running along x lie one pixel row apart: with 8 float-float
-// instances a pixel takes 64 bytes, half of a bank line, and the swap puts such pairs in different
-// halves (as for pixels one column apart) instead of in the same one.
-__host__ __device__ inline int tile_slot(int q, int TX) { return q ^ ((q / TX) & 1); }
+// A staged row in shared memory and a lane's part of it.
+template <typename TW, int IC>
+struct Staged;
 
-template <typename TW, int VV>
-__global__ void __launch_bounds__(kThreads) kbx_tile_apply(BDims D, TiledA T, BBulkX<TW> X, BSmall S, int IC,
-                                                           float2* __restrict__ part) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    TW* ws = reinterpret_cast<TW*>(smem_raw);   // [TX * TY][IC]
-    const int B = D.B, nch = B / IC, G = IC / VV, NSL = kThreads / G;
-    const int t = (int)(blockIdx.x / nch), c = (int)(blockIdx.x % nch);
-    const int ig = threadIdx.x % G, sl = threadIdx.x / G;
-    const int b0 = c * IC + ig * VV;
-    const TW* wb[VV];
-    bool same = true;
-#pragma unroll
-    for (int v = 0; v < VV; ++v) {
-        const DevScalars& sc = S.sc[b0 + v];
-        wb[v] = (!sc.stop && sc.d < D.dmax) ? X.W + (size_t)sc.d * D.n * B + b0 + v : nullptr;
-        same = same && wb[v] && S.sc[b0 + v].d == S.sc[b0].d;
+// float-float: pairs of instances as (hi0, hi1, lo0, lo1).  With 16 instances a row fills all banks; the
+// eight lanes of a load phase belong to two rows, and those of the odd one take the row's upper half
+// first, so that the phase touches every bank once.
+template <int IC>
+struct Staged<float2, IC> {
+    using LN = Lanes<IC>;
+    static constexpr int kRow = IC * 8;
+    int first;    // instance of accumulator 0
+    int second;   // of accumulator 1 (VV = 4)
+    const unsigned char *p0, *p1;
+    __device__ __forceinline__ Staged(const unsigned char* base, int j, int row) {
+        if constexpr (LN::VV == 4) {
+            const int c0 = j + ((row & 1) ? LN::G : 0), c1 = j + ((row & 1) ? 0 : LN::G);
+            first = 2 * c0;
+            second = 2 * c1;
+        } else {
+            first = second = LN::VV * j;
+        }
+        p0 = base + first * 8;
+        p1 = base + second * 8;
     }
+    __device__ __forceinline__ int inst(int v) const { return (v < 2 ? first : second) + (v & 1); }
+    __device__ __forceinline__ void add(Dot2x2 (&d)[LN::NP], uint32_t slot, float c) const {
+        const f32x2 cc = pack2(c, c);
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p0 + slot * kRow);
+        d[0].add_prod2(cc, v.x, v.y);
+        if constexpr (LN::NP == 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(p1 + slot * kRow);
+            d[1].add_prod2(cc, w.x, w.y);
+        }
+    }
+    __device__ __forceinline__ void add_both(Dot2x2& d, uint32_t s0, uint32_t s1, float c0, float c1) const {
+        const float2 a = *reinterpret_cast<const float2*>(p0 + s0 * kRow), b = *reinterpret_cast<const float2*>(p0 + s1 * kRow);
+        d.add_prod2(pack2(c0, c1), pack2(a.x, b.x), pack2(a.y, b.y));
+    }
+    // the lane's instances of row `slot`, v[k] instance inst(k)
+    __device__ __forceinline__ void put(unsigned char* base, int slot, const float2 (&v)[LN::VV]) const {
+        if constexpr (LN::VV == 1) {
+            *reinterpret_cast<float2*>(base + slot * kRow) = v[0];
+        } else {
+            *reinterpret_cast<float4*>(base + slot * kRow + first * 8) = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
+            if constexpr (LN::VV == 4)
+                *reinterpret_cast<float4*>(base + slot * kRow + second * 8) = make_float4(v[2].x, v[3].x, v[2].y, v[3].y);
+        }
+    }
+};
+
+// FP32 basis: plain values, a lane's VV next to each other
+template <int IC>
+struct Staged<float, IC> {
+    using LN = Lanes<IC>;
+    static constexpr int kRow = IC * 4;
+    int first;
+    const unsigned char* p0;
+    __device__ __forceinline__ Staged(const unsigned char* base, int j, int) : first(LN::VV * j), p0(base + LN::VV * j * 4) {}
+    __device__ __forceinline__ int inst(int v) const { return first + v; }
+    __device__ __forceinline__ void add(Dot2x2 (&d)[LN::NP], uint32_t slot, float c) const {
+        const f32x2 cc = pack2(c, c);
+        if constexpr (LN::NP == 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p0 + slot * kRow);
+            d[0].add_prod(cc, v.x);
+            d[1].add_prod(cc, v.y);
+        } else {
+            d[0].add_prod(cc, *reinterpret_cast<const f32x2*>(p0 + slot * kRow));
+        }
+    }
+    __device__ __forceinline__ void add_both(Dot2x2& d, uint32_t s0, uint32_t s1, float c0, float c1) const {
+        d.add_prod(pack2(c0, c1), pack2(*reinterpret_cast<const float*>(p0 + s0 * kRow), *reinterpret_cast<const float*>(p0 + s1 * kRow)));
+    }
+    __device__ __forceinline__ void put(unsigned char* base, int slot, const float (&v)[LN::VV]) const {
+#pragma unroll
+        for (int k = 0; k < LN::VV; ++k) *reinterpret_cast<float*>(base + slot * kRow + (first + k) * 4) = v[k];
+    }
+};
+
+// A row's entry pairs are read as one stream with those of the rows that the lane takes after it: two
+// pairs (four entries) at a time, the next two on their way while the present ones are added, also
+// from one row to the next.  The loads run two pairs past a row's last ones at most, into the next group
+// or into the filling behind the last one (kTileAhead).
+struct Entries {
+    uint4 a, b;
+    __device__ __forceinline__ void load(const uint4* __restrict__ ent, int pair) {
+        const uint4* q = ent + (size_t)pair * 4;
+        a = __ldg(q);
+        b = __ldg(q + 4);
+    }
+};
+
+// The next row's entries (pairs [beg, end) of its group) into L2, a line per lane: the first CTA that
+// comes to a tile would otherwise wait for HBM at every row (2.04 -> 2.01 ms per pass, 512^2 at 64).
+__device__ __forceinline__ void entries_to_l2(const uint4* ent, int beg, int end, int k) {
+    if (beg + 2 * k < end) asm volatile("prefetch.global.L2 [%0];" ::"l"(ent + (size_t)(beg + 2 * k) * 4));
+}
+
+template <typename TW, int IC>
+__device__ __forceinline__ void add_pair(Dot2x2 (&d)[Lanes<IC>::NP], const Staged<TW, IC>& st, const uint4& e) {
+    if constexpr (Lanes<IC>::VV == 1) {
+        st.add_both(d[0], e.x, e.y, __uint_as_float(e.z), __uint_as_float(e.w));
+    } else {
+        st.add(d, e.x, __uint_as_float(e.z));
+        st.add(d, e.y, __uint_as_float(e.w));
+    }
+}
+
+// Pairs [beg, end) of a row into acc, in blocks of kDot2Block terms (ff.cuh); cur holds the pairs beg
+// and beg + 1 and leaves with those of the next row, from `next` on.  FIRST: acc is still 0.
+template <bool FIRST, typename TW, int IC>
+__device__ __forceinline__ void add_row(Dot2x2 (&acc)[Lanes<IC>::NP], const Staged<TW, IC>& st, Entries& cur,
+                                        const uint4* __restrict__ ent, int beg, int end, int next) {
+    constexpr int NP = Lanes<IC>::NP, PB = kDot2Block / 2;
+    static_assert(PB % 4 == 0, "blocks of whole double steps");
+    if (beg == end) {
+        cur.load(ent, next);
+        return;
+    }
+    for (int kb = beg; kb < end; kb += PB) {
+        const int ke = min(end, kb + PB);
+        Dot2x2 blk[NP];
+        for (int k = kb; k < ke; k += 4) {
+            Entries nxt;
+            nxt.load(ent, k + 2 < end ? k + 2 : next);
+            add_pair<TW, IC>(blk, st, cur.a);
+            if (k + 1 < ke) add_pair<TW, IC>(blk, st, cur.b);
+            if (k + 2 < ke) {
+                cur.load(ent, k + 4 < end ? k + 4 : next);
+                add_pair<TW, IC>(blk, st, nxt.a);
+                if (k + 3 < ke) add_pair<TW, IC>(blk, st, nxt.b);
+            } else {
+                cur = nxt;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            if (FIRST && kb == beg) acc[i] = blk[i];
+            else acc[i].merge(blk[i]);
+        }
+    }
+}
+
+// A batch of one: the sums of the first and of the second entries
+__device__ __forceinline__ Dot2 both_halves(const Dot2x2& a) {
+    Dot2 d = a.half(0);
+    d.merge(a.half(1));
+    return d;
+}
+
+}  // namespace
+
+// ------------------------------------------------------------------------------- u = A w
+// CTA (tile, IC instances)
+template <typename TW, int IC>
+__global__ void __launch_bounds__(Lanes<IC>::threads, IC >= 16 ? 3 : 2) kbx_tile_apply(BDims D, TiledA T, BBulkX<TW> X, BSmall S,
+                                                              int split, float2* __restrict__ part) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    using LN = Lanes<IC>;
+    constexpr int rows = LN::threads / LN::G;   // segments that the CTA walks at a time
+    const int B = D.B, nch = B / IC;
+    const int bid = (int)blockIdx.x / split, sp = (int)blockIdx.x - bid * split;
+    const int t = T.order[bid / nch], c = bid % nch;
+    const int row = threadIdx.x / LN::G;
+    const Staged<TW, IC> st(smem_raw, threadIdx.x % LN::G, row);
+    const TW* wb[LN::VV];
+    bool any = false;
+#pragma unroll
+    for (int v = 0; v < LN::VV; ++v) {
+        const int b = c * IC + st.inst(v);
+        const DevScalars& sc = S.sc[b];
+        wb[v] = (!sc.stop && sc.d < D.dmax) ? X.W + (size_t)sc.d * D.n * B + b : nullptr;
+        any = any || wb[v];
+    }
+    if (!__syncthreads_or(any)) return;
     const int tpf = T.ntx * T.nty;
     const int f = t / tpf, rt = t - f * tpf, ty = rt / T.ntx, tx = rt - ty * T.ntx;
     const int npx = T.TX * T.TY;
     const int64_t fbase = (int64_t)f * T.nx * T.ny;
-    for (int q = sl; q < npx; q += NSL) {
+    for (int q = row; q <= npx; q += rows) {   // slot npx holds 0
         const int py = q / T.TX, px = q - py * T.TX;
         const int iy = ty * T.TY + py, ix = tx * T.TX + px;
-        TW v[VV];
-        const bool in = iy < T.ny && ix < T.nx;
+        const bool in = q < npx && iy < T.ny && ix < T.nx;
         const int64_t off = (fbase + (int64_t)iy * T.nx + ix) * B;
-        if (in && same && VV * sizeof(TW) == 16) {
-            const float4 f4 = __ldcg(reinterpret_cast<const float4*>(wb[0] + off));
-            *reinterpret_cast<float4*>(v) = f4;
-        } else {
+        TW v[LN::VV];
 #pragma unroll
-            for (int k = 0; k < VV; ++k) v[k] = (in && wb[k]) ? __ldcg(wb[k] + off) : tzero<TW>();
-        }
-        const int qs = tile_slot(q, T.TX);
-#pragma unroll
-        for (int k = 0; k < VV; ++k) ws[qs * IC + ig * VV + k] = v[k];
+        for (int k = 0; k < LN::VV; ++k) v[k] = (in && wb[k]) ? __ldcg(wb[k] + off) : TW{};
+        st.put(smem_raw, q < npx ? tile_slot(q, T.TX) : npx, v);
     }
     __syncthreads();
-    const int s0 = T.tile_seg[t], s1 = T.tile_seg[t + 1];
-    for (int s = s0 + sl; s < s1; s += NSL) {
-        const int e0 = T.seg_ent[s], e1 = T.seg_ent[s + 1];
-        Dot2 a[VV];
-#pragma unroll 4
-        for (int k = e0; k < e1; ++k) {
-            const uint2 en = __ldg(T.ent + k);
-            const float av = __uint_as_float(en.y);
-            TW wv[VV];
-            if constexpr (VV * sizeof(TW) == 16) {
-                *reinterpret_cast<float4*>(wv) = *reinterpret_cast<const float4*>(ws + (int)en.x * IC + ig * VV);
-            } else {
+    // segments s, s + step, ... of the tile: (beg, end) of the present one and of the next
+    const int s1 = T.tile_grp[t + 1] * 4, step = rows * split;
+    int s = T.tile_grp[t] * 4 + sp * rows + row;
+    if (s >= s1) return;
+    const uint4* ent = T.ent + (s & 3);
+    auto group = [&](int q, int& beg, int& end) {
+        const int g = min(q, s1 - 1) >> 2;
+        beg = T.goff[g];
+        end = T.goff[g + 1];
+    };
+    int beg, end, nbeg, nend;
+    group(s, beg, end);
+    group(s + step, nbeg, nend);
+    Entries cur;
+    cur.load(ent, beg);
+    for (; s < s1; s += step) {
+        int fbeg, fend;
+        group(s + 2 * step, fbeg, fend);
+        if constexpr (IC == 16) entries_to_l2(T.ent, nbeg, nend, threadIdx.x & 15);
+        Dot2x2 a[LN::NP];
+        add_row<true, TW, IC>(a, st, cur, ent, beg, end, nbeg);
+        beg = nbeg;
+        end = nend;
+        nbeg = fbeg;
+        nend = fend;
+        float2* dst = part + (size_t)s * B + c * IC;
+        if constexpr (LN::VV == 1) {
+            dst[0] = both_halves(a[0]).value();
+        } else {
 #pragma unroll
-                for (int v = 0; v < VV; ++v) wv[v] = ws[(int)en.x * IC + ig * VV + v];
+            for (int i = 0; i < LN::NP; ++i) {
+                ulonglong2 o;
+                a[i].value(o.x, o.y);
+                *reinterpret_cast<ulonglong2*>(dst + st.inst(2 * i)) = o;
             }
-#pragma unroll
-            for (int v = 0; v < VV; ++v) tacc(a[v], av, wv[v]);
         }
-        float2* dst = part + (size_t)T.seg_slot[s] * B + b0;
-#pragma unroll
-        for (int v = 0; v < VV; ++v) dst[v] = a[v].value();
     }
 }
 
-// u_i = sum over the ray's segments (in order) of the partials -> column d_i of AW.
-template <typename TW>
+// u_i = sum over the ray's segments, in the order of the row's entries, of the partials -> column
+// d_i of AW.  NB = 2: a thread takes two instances, partials as (hi0, hi1, lo0, lo1).
+template <typename TW, int NB>
 __global__ void __launch_bounds__(kThreads) kbx_seg_reduce(BDims D, TiledA T, BBulkX<TW> X, BSmall S,
                                                            const float2* __restrict__ part) {
-    const int B = D.B;
-    const int b = threadIdx.x & (B - 1);
-    const DevScalars& sc = S.sc[b];
-    if (sc.stop || sc.d >= D.dmax) return;
-    float2* out = X.AW + (size_t)sc.d * D.m * B + b;
-    for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t < D.m * B; t += gstride()) {
-        const int64_t r = qdiv(t, B);
-        Dot2 a;
-        for (int s = T.ray_slot[r]; s < T.ray_slot[r + 1]; ++s) {
-            const float2 v = __ldcg(part + (size_t)s * B + b);
-            a.add2(v.x, v.y);
+    const int B = D.B, H = B / NB;
+    const int b = (threadIdx.x & (H - 1)) * NB;
+    float2* out[NB];
+    bool any = false;
+#pragma unroll
+    for (int v = 0; v < NB; ++v) {
+        const DevScalars& sc = S.sc[b + v];
+        out[v] = (!sc.stop && sc.d < D.dmax) ? X.AW + (size_t)sc.d * D.m * B + b + v : nullptr;
+        any = any || out[v];
+    }
+    if (!any) return;
+    for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t < D.m * H; t += gstride()) {
+        const int64_t r = qdiv(t, H);
+        const int k0 = T.ray_ptr[r], k1 = T.ray_ptr[r + 1];
+        if constexpr (NB == 2) {
+            Dot2x2 a;
+#pragma unroll 4
+            for (int k = k0; k < k1; ++k) {
+                const float4 f = __ldcs(reinterpret_cast<const float4*>(part + (size_t)T.ray_seg[k] * B + b));
+                a.accumulate(pack2(f.x, f.y), pack2(f.z, f.w));
+                if ((k - k0) % 4 == 3) a.renorm();   // ff.cuh: free, the loads set the pace
+            }
+            if (out[0]) out[0][r * B] = a.half(0).value();
+            if (out[NB - 1]) out[NB - 1][r * B] = a.half(1).value();
+        } else {
+            Dot2 a;
+#pragma unroll 4
+            for (int k = k0; k < k1; ++k) {
+                const float2 v = __ldcs(part + (size_t)T.ray_seg[k] * B + b);
+                a.add2(v.x, v.y);
+                if ((k - k0) % 4 == 3) a.renorm();
+            }
+            if (out[0]) out[0][r * B] = a.value();
         }
-        out[r * B] = a.value();
     }
 }
 
-int tile_instances(const BDims& D, size_t welem) {
-    return std::min(D.B, D.tile_ic > 0 ? D.tile_ic : (welem == 4 ? 16 : 8));
+// --------------------------------------------------------- r = A^T e + lambda L^T L x
+// CTA (tile of 16 x TY pixels, IC instances); a thread holds PP pixels (u rows + its row) of the tile.
+// out == nullptr: appended as column d_i of W_i (rounded to TW); otherwise written to out.
+template <int IC, int TY>
+struct GradShape {
+    static constexpr int px = kTileTX * TY, threads = std::min(Lanes<IC>::threads, px * Lanes<IC>::G);
+    static constexpr int rows = threads / Lanes<IC>::G, PP = px / rows;
+};
+
+template <typename TW, int IC, int TY>
+__global__ void __launch_bounds__(GradShape<IC, TY>::threads, IC >= 16 ? 3 : 1024 / GradShape<IC, TY>::threads)
+    kbx_tile_gradient(BDims D, TiledT T, DevL L, BBulkX<TW> X, BSmall S, float2* out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    using LN = Lanes<IC>;
+    constexpr int rows = GradShape<IC, TY>::rows, PP = GradShape<IC, TY>::PP;
+    const int B = D.B, nch = B / IC;
+    const int t = T.order[blockIdx.x / nch], c = (int)(blockIdx.x % nch);
+    const int row = threadIdx.x / LN::G;
+    const Staged<float2, IC> st(smem_raw, threadIdx.x % LN::G, row);
+    bool any = false;
+#pragma unroll
+    for (int v = 0; v < LN::VV; ++v) {
+        DevScalars& sc = S.sc[c * IC + st.inst(v)];
+        if (sc.stop) continue;
+        if (!out && sc.d >= D.dmax) {
+            if (t == 0 && row == 0) {
+                sc.status = ST_FULL;
+                sc.stop = 1;
+            }
+            continue;
+        }
+        any = true;
+    }
+    if (!__syncthreads_or(any)) return;
+    Dot2x2 acc[PP][LN::NP];
+    // Rows of entries of this lane: pixel u of stage k is group g0 + (k PP + u) rows / 4
+    const int ray1 = T.tile_ray[t + 1], stages = T.tile_stage[t + 1] - T.tile_stage[t];
+    const uint4* ent = T.ent + (row & 3);
+    int g = T.tile_stage[t] * (kTileTX * TY / 4) + (row >> 2);
+    const int glast = g + (stages * PP - 1) * (rows / 4);
+    int beg = 0, end = 0, nbeg = 0, nend = 0;
+    Entries cur{};
+    if (stages) {
+        beg = T.goff[g];
+        end = T.goff[g + 1];
+        g = min(g + rows / 4, glast);
+        nbeg = T.goff[g];
+        nend = T.goff[g + 1];
+        cur.load(ent, beg);
+    }
+    for (int r0 = T.tile_ray[t]; r0 < ray1; r0 += T.stage) {
+        const int nr = min(T.stage, ray1 - r0);
+        __syncthreads();   // the stage before has been read
+#pragma unroll 4
+        for (int q = row; q <= nr; q += rows) {
+            float2 v[LN::VV] = {};
+            if (q < nr) {
+                const float2* src = X.e + (size_t)T.ray[r0 + q] * B + c * IC;
+                if constexpr (LN::VV == 1) {
+                    v[0] = __ldcg(src);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < LN::NP; ++i) {
+                        const float4 f = __ldcg(reinterpret_cast<const float4*>(src + st.inst(2 * i)));
+                        v[2 * i] = make_float2(f.x, f.y);
+                        v[2 * i + 1] = make_float2(f.z, f.w);
+                    }
+                }
+            }
+            st.put(smem_raw, q < nr ? q : T.stage, v);   // slot T.stage holds 0
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < PP; ++u) {
+            g = min(g + rows / 4, glast);
+            const int fbeg = T.goff[g], fend = T.goff[g + 1];
+            if constexpr (IC == 16) entries_to_l2(T.ent, nbeg, nend, threadIdx.x & 15);
+            add_row<false, float2, IC>(acc[u], st, cur, ent, beg, end, nbeg);
+#pragma unroll
+            for (int i = 0; i < LN::NP; ++i) acc[u][i].renorm();   // once per stage (ff.cuh)
+            beg = nbeg;
+            end = nend;
+            nbeg = fbeg;
+            nend = fend;
+        }
+    }
+    const int tpf = T.ntx * T.nty;
+    const int f = t / tpf, rt = t - f * tpf, ty = rt / T.ntx, tx = rt - ty * T.ntx;
+#pragma unroll
+    for (int u = 0; u < PP; ++u) {
+        const int loc = u * rows + row;
+        const int iy = ty * TY + loc / kTileTX, ix = tx * kTileTX + loc % kTileTX;
+        if (iy >= T.ny || ix >= T.nx) continue;
+        const int64_t i = ((int64_t)f * T.ny + iy) * T.nx + ix;
+#pragma unroll
+        for (int v = 0; v < LN::VV; ++v) {
+            const int b = c * IC + st.inst(v);
+            const DevScalars& sc = S.sc[b];
+            const int d = sc.d;
+            if (sc.stop || (!out && d >= D.dmax)) continue;
+            Dot2 a = LN::VV == 1 ? both_halves(acc[u][0]) : acc[u][v / 2].half(v & 1);
+            Dot2 lt;
+            ff_ltl_row(lt, L, i, StridedW<float2>{X.x + b, B});
+            const float2 ltv = lt.value(), lam = X.lam2[b];
+            a.add_prod22(lam.x, lam.y, ltv.x, ltv.y);
+            if (out) out[i * B + b] = a.value();
+            else store_w(X.W + ((size_t)d * D.n + i) * B + b, a);
+        }
+    }
 }
 
-size_t tile_smem(const TiledA& T, const BDims& D, size_t welem) {
-    return (size_t)T.TX * T.TY * tile_instances(D, welem) * welem;
+// ------------------------------------------------------------------------------ launchers
+int tile_instances(const BDims& D) { return std::min(D.B, D.tile_ic > 0 ? D.tile_ic : kTileInst); }
+
+template <typename K>
+static cudaError_t tile_smem_limit(K k, size_t smem) {
+    return smem > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
 }
 
-template <typename TW, int VV>
-static cudaError_t tile_apply_vv(const BDims& D, const TiledA& T, const BBulkX<TW>& X, const BSmall& S, float2* part,
+template <typename TW, int IC>
+static cudaError_t tile_apply_ic(const BDims& D, const TiledA& T, const BBulkX<TW>& X, const BSmall& S, float2* part,
                                  cudaStream_t st) {
-    const int IC = tile_instances(D, sizeof(TW));
-    const size_t smem = tile_smem(T, D, sizeof(TW));
-    auto k = kbx_tile_apply<TW, VV>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    const int64_t grid = (int64_t)T.ntiles * (D.B / IC);
-    k<<<(unsigned)grid, kThreads, smem, st>>>(D, T, X, S, IC, part);
+    const size_t smem = (size_t)(T.TX * T.TY + 1) * IC * sizeof(TW);
+    auto k = kbx_tile_apply<TW, IC>;
+    cudaError_t e = tile_smem_limit(k, smem);
+    if (e != cudaSuccess) return e;
+    // A tile's segments go to `split` CTAs (each stages the tile) until there are eight rounds of CTAs:
+    // with 4.5 rounds, 512^2 at 64 instances, the last one leaves a tenth of the chip's time unused.
+    // Eight segments or more remain for every lane, against the staging.
+    const int64_t ctas = (int64_t)T.ntiles * (D.B / IC), rows = Lanes<IC>::threads / Lanes<IC>::G;
+    const int64_t want = std::min<int64_t>(4, (8 * 152 * 3 + ctas - 1) / ctas), most = T.npart / (T.ntiles * rows * 8);
+    const int split = (int)std::max<int64_t>(1, std::min(want, most));
+    k<<<(unsigned)(ctas * split), Lanes<IC>::threads, smem, st>>>(D, T, X, S, split, part);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    constexpr int NB = IC == 1 ? 1 : 2;
+    const int64_t rb = (D.m * (D.B / NB) + kThreads - 1) / kThreads;
+    kbx_seg_reduce<TW, NB><<<(int)std::max<int64_t>(1, std::min<int64_t>(rb, 8 * 152)), kThreads, 0, st>>>(D, T, X, S, part);
     return cudaGetLastError();
 }
 
 template <typename TW>
 cudaError_t launchbx_tile_apply(const BDims& D, const TiledA& T, const BBulkX<TW>& X, const BSmall& S, float2* part,
                                 cudaStream_t st) {
-    constexpr int VW = 16 / (int)sizeof(TW);
-    const int IC = tile_instances(D, sizeof(TW));
-    cudaError_t e = IC >= VW ? tile_apply_vv<TW, VW>(D, T, X, S, part, st) : tile_apply_vv<TW, 1>(D, T, X, S, part, st);
+    switch (tile_instances(D)) {
+        case 1: return tile_apply_ic<TW, 1>(D, T, X, S, part, st);
+        case 2: return tile_apply_ic<TW, 2>(D, T, X, S, part, st);
+        case 4: return tile_apply_ic<TW, 4>(D, T, X, S, part, st);
+        case 8: return tile_apply_ic<TW, 8>(D, T, X, S, part, st);
+        default: return tile_apply_ic<TW, 16>(D, T, X, S, part, st);
+    }
+}
+
+template <typename TW, int IC, int TY>
+static cudaError_t tile_gradient_ty(const BDims& D, const TiledT& T, const DevL& L, const BBulkX<TW>& X, const BSmall& S,
+                                    float2* out, cudaStream_t st) {
+    const size_t smem = (size_t)(T.stage + 1) * IC * sizeof(float2);
+    auto k = kbx_tile_gradient<TW, IC, TY>;
+    const cudaError_t e = tile_smem_limit(k, smem);
     if (e != cudaSuccess) return e;
-    int64_t rb = (D.m * D.B + kThreads - 1) / kThreads;
-    if (rb > 8 * 152) rb = 8 * 152;
-    kbx_seg_reduce<TW><<<(int)(rb < 1 ? 1 : rb), kThreads, 0, st>>>(D, T, X, S, part);
+    k<<<(unsigned)((int64_t)T.ntiles * (D.B / IC)), GradShape<IC, TY>::threads, smem, st>>>(D, T, L, X, S, out);
     return cudaGetLastError();
 }
 
-template cudaError_t launchbx_tile_apply<float>(const BDims&, const TiledA&, const BBulkX<float>&, const BSmall&,
-                                                float2*, cudaStream_t);
-template cudaError_t launchbx_tile_apply<float2>(const BDims&, const TiledA&, const BBulkX<float2>&, const BSmall&,
-                                                 float2*, cudaStream_t);
-
-// ------------------------------------------------------------------------ host re-blocking
-// Rows of A (rp, ci, val on the device) cut into (row, tile) segments for an image of nt frames
-// of ny x nx pixels (unknown index f nx ny + iy nx + ix).  Device arrays go to `allocs`.
-int build_tiles(const int32_t* d_rp, const int32_t* d_ci, const float* d_val, int64_t m, int64_t n, int64_t nnz,
-                int nx, int ny, int nt, int TX, int TY, TiledA& T, std::vector<void*>& allocs, cudaStream_t st,
-                std::string* why) {
-    if ((int64_t)nx * ny * nt != n || TX * TY > 65536 || TX % 2 != 0 || nnz >= ((int64_t)1 << 31)) {
-        *why = "tiled operator: geometry does not match the unknowns";
-        return SGKS_ERR_INVALID;
-    }
-    std::vector<int32_t> rp((size_t)m + 1), ci((size_t)nnz);
-    std::vector<float> val((size_t)nnz);
-    cudaError_t e = cudaMemcpyAsync(rp.data(), d_rp, sizeof(int32_t) * (m + 1), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && nnz)
-        e = cudaMemcpyAsync(ci.data(), d_ci, sizeof(int32_t) * nnz, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && nnz)
-        e = cudaMemcpyAsync(val.data(), d_val, sizeof(float) * nnz, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-        *why = std::string("tiled operator: ") + cudaGetErrorString(e);
-        return SGKS_ERR_CUDA;
-    }
-    const int ntx = (nx + TX - 1) / TX, nty = (ny + TY - 1) / TY;
-    const int64_t tpf = (int64_t)ntx * nty, ntiles = tpf * nt;
-    if (ntiles >= ((int64_t)1 << 31)) {
-        *why = "tiled operator: too many tiles";
-        return SGKS_ERR_INVALID;
-    }
-    const int64_t fr = (int64_t)nx * ny;
-    std::vector<int32_t> tile_of((size_t)nnz), loc_of((size_t)nnz);
-    for (int64_t k = 0; k < nnz; ++k) {
-        const int64_t col = ci[(size_t)k];
-        const int64_t f = col / fr, r = col - f * fr, iy = r / nx, ix = r - iy * nx;
-        tile_of[(size_t)k] = (int32_t)(f * tpf + (iy / TY) * ntx + ix / TX);
-        // staged w is laid out in checkerboard order (tile_slot): neighbouring pixels in x and
-        // in y fall in different halves of the 128-byte bank line
-        loc_of[(size_t)k] = tile_slot((iy % TY) * TX + ix % TX, TX);
-    }
-    // pass 1: per row, entries stably ordered by tile; segments are the runs; count per tile
-    std::vector<int32_t> order((size_t)nnz);
-    std::iota(order.begin(), order.end(), 0);
-    std::vector<int32_t> ray_slot((size_t)m + 1, 0);
-    std::vector<int64_t> tile_nseg((size_t)ntiles, 0), tile_nent((size_t)ntiles, 0);
-    int64_t nseg = 0;
-    for (int64_t r = 0; r < m; ++r) {
-        const int32_t a = rp[(size_t)r], z = rp[(size_t)r + 1];
-        std::stable_sort(order.begin() + a, order.begin() + z,
-                         [&](int32_t p, int32_t q) { return tile_of[(size_t)p] < tile_of[(size_t)q]; });
-        ray_slot[(size_t)r] = (int32_t)nseg;
-        for (int32_t k = a; k < z; ++k) {
-            const int32_t tl = tile_of[(size_t)order[(size_t)k]];
-            if (k == a || tl != tile_of[(size_t)order[(size_t)k - 1]]) {
-                ++nseg;
-                ++tile_nseg[(size_t)tl];
-            }
-            ++tile_nent[(size_t)tl];
-        }
-    }
-    ray_slot[(size_t)m] = (int32_t)nseg;
-    if (nseg >= ((int64_t)1 << 31)) {
-        *why = "tiled operator: too many segments";
-        return SGKS_ERR_INVALID;
-    }
-    // pass 2: segments and entries in tile-major order (a tile's segments in row order)
-    std::vector<int32_t> tile_seg((size_t)ntiles + 1, 0);
-    std::vector<int64_t> tile_ent((size_t)ntiles + 1, 0);
-    for (int64_t t = 0; t < ntiles; ++t) {
-        tile_seg[(size_t)t + 1] = tile_seg[(size_t)t] + (int32_t)tile_nseg[(size_t)t];
-        tile_ent[(size_t)t + 1] = tile_ent[(size_t)t] + tile_nent[(size_t)t];
-    }
-    std::vector<int32_t> seg_fill(tile_seg.begin(), tile_seg.end() - 1);
-    std::vector<int64_t> ent_fill(tile_ent.begin(), tile_ent.end() - 1);
-    std::vector<int32_t> seg_ent((size_t)nseg + 1, 0), seg_slot((size_t)nseg, 0);
-    std::vector<uint32_t> ent((size_t)nnz * 2);   // (local pixel, value bits) per entry
-    int64_t slot = 0;
-    for (int64_t r = 0; r < m; ++r) {
-        const int32_t a = rp[(size_t)r], z = rp[(size_t)r + 1];
-        int32_t k = a;
-        while (k < z) {
-            const int32_t tl = tile_of[(size_t)order[(size_t)k]];
-            int32_t k2 = k;
-            while (k2 < z && tile_of[(size_t)order[(size_t)k2]] == tl) ++k2;
-            const int32_t gs = seg_fill[(size_t)tl]++;
-            int64_t pos = ent_fill[(size_t)tl];
-            seg_ent[(size_t)gs] = (int32_t)pos;
-            seg_slot[(size_t)gs] = (int32_t)slot++;
-            for (int32_t q = k; q < k2; ++q) {
-                const int32_t src = order[(size_t)q];
-                uint32_t vb;
-                memcpy(&vb, &val[(size_t)src], sizeof(vb));
-                ent[(size_t)pos * 2] = (uint32_t)loc_of[(size_t)src];
-                ent[(size_t)pos * 2 + 1] = vb;
-                ++pos;
-            }
-            ent_fill[(size_t)tl] = pos;
-            k = k2;
-        }
-    }
-    seg_ent[(size_t)nseg] = (int32_t)nnz;
-    // device copies
-    auto up = [&](const void* host, size_t bytes, void** dptr) -> cudaError_t {
-        void* p = nullptr;
-        cudaError_t e2 = cudaMalloc(&p, bytes ? bytes : 16);
-        if (e2 != cudaSuccess) return e2;
-        allocs.push_back(p);
-        *dptr = p;
-        return bytes ? cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, st) : cudaSuccess;
-    };
-    void *p1, *p2, *p3, *p4, *p5;
-    e = up(tile_seg.data(), sizeof(int32_t) * tile_seg.size(), &p1);
-    if (e == cudaSuccess) e = up(seg_ent.data(), sizeof(int32_t) * seg_ent.size(), &p2);
-    if (e == cudaSuccess) e = up(seg_slot.data(), sizeof(int32_t) * seg_slot.size(), &p3);
-    if (e == cudaSuccess) e = up(ray_slot.data(), sizeof(int32_t) * ray_slot.size(), &p4);
-    if (e == cudaSuccess) e = up(ent.data(), sizeof(uint32_t) * ent.size(), &p5);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the host vectors die on return
-    if (e != cudaSuccess) {
-        *why = std::string("tiled operator: ") + cudaGetErrorString(e);
-        return e == cudaErrorMemoryAllocation ? SGKS_ERR_NOMEM : SGKS_ERR_CUDA;
-    }
-    T = TiledA{};
-    T.TX = TX;
-    T.TY = TY;
-    T.nx = nx;
-    T.ny = ny;
-    T.nt = nt;
-    T.ntx = ntx;
-    T.nty = nty;
-    T.ntiles = (int)ntiles;
-    T.nseg = nseg;
-    T.tile_seg = (const int32_t*)p1;
-    T.seg_ent = (const int32_t*)p2;
-    T.seg_slot = (const int32_t*)p3;
-    T.ray_slot = (const int32_t*)p4;
-    T.ent = (const uint2*)p5;
-    return SGKS_OK;
+template <typename TW, int IC>
+static cudaError_t tile_gradient_ic(const BDims& D, const TiledT& T, const DevL& L, const BBulkX<TW>& X, const BSmall& S,
+                                    float2* out, cudaStream_t st) {
+    return T.TY == 8 ? tile_gradient_ty<TW, IC, 8>(D, T, L, X, S, out, st)
+                     : tile_gradient_ty<TW, IC, 16>(D, T, L, X, S, out, st);
 }
+
+template <typename TW>
+cudaError_t launchbx_tile_gradient(const BDims& D, const TiledT& T, const DevL& L, const BBulkX<TW>& X, const BSmall& S,
+                                   float2* out, cudaStream_t st) {
+    switch (std::min(D.B, kTileInst)) {
+        case 1: return tile_gradient_ic<TW, 1>(D, T, L, X, S, out, st);
+        case 2: return tile_gradient_ic<TW, 2>(D, T, L, X, S, out, st);
+        case 4: return tile_gradient_ic<TW, 4>(D, T, L, X, S, out, st);
+        case 8: return tile_gradient_ic<TW, 8>(D, T, L, X, S, out, st);
+        default: return tile_gradient_ty<TW, 16, 8>(D, T, L, X, S, out, st);   // T is built for the largest group
+    }
+}
+
+#define SGKS_INST_TILES(TW)                                                                                         \
+    template cudaError_t launchbx_tile_apply<TW>(const BDims&, const TiledA&, const BBulkX<TW>&, const BSmall&,     \
+                                                 float2*, cudaStream_t);                                            \
+    template cudaError_t launchbx_tile_gradient<TW>(const BDims&, const TiledT&, const DevL&, const BBulkX<TW>&,    \
+                                                    const BSmall&, float2*, cudaStream_t);
+SGKS_INST_TILES(float)
+SGKS_INST_TILES(float2)
 
 }  // namespace sgks

@@ -291,7 +291,8 @@ struct GroupX : GroupBase {
     SketchCSR SK{};
     int io_dt = SGKS_F32;       // element type of the caller's b, x_true and x_out
     TiledA T{};                 // pixel tiles of a CSR A (ntiles = 0: the CSR-row kernel)
-    float2* part = nullptr;     // [nseg][B] partial sums of the tiled forward pass
+    TiledT Tt{};                // the same of A^T
+    float2* part = nullptr;     // [npart][B] partial sums of the tiled forward pass
     SketchLChunks LC{};         // S_L in column chunks of L w
     float2* lpart = nullptr;    // [nchunks][s][B] partial sums of S_L L w
 
@@ -304,6 +305,11 @@ struct GroupX : GroupBase {
         return e;
     }
 
+    cudaError_t gradient(const BBulkX<TW>& Xg, float2* out) {
+        return Tt.ntiles ? launchbx_tile_gradient<TW>(D, Tt, L, Xg, S, out, st)
+                         : launchbx_gradient<TW>(D, A, L, Xg, S, out, st);
+    }
+
     cudaError_t small_append() {
         cudaError_t e = cudaSuccess;
         RUNC(BK_QR_APPEND, 1, launch_qr_append(Ds, Small{}, st, Sarr, D.B));
@@ -314,7 +320,7 @@ struct GroupX : GroupBase {
     cudaError_t refine() {
         cudaError_t e = cudaSuccess;
         RUNC(BK_COMBINE_REFINE, 2, launchbx_combine<TW>(D, X, S, 0, st));
-        RUNC(BK_GRAD_REFINE, 1, launchbx_gradient<TW>(D, A, L, X, S, X.r, st));
+        RUNC(BK_GRAD_REFINE, 1, gradient(X, X.r));
         RUNC(BK_GRAD_REFINE, 1, launchbx_wtr<TW>(D, X, S, X.r, st));
         RUNC(BK_REFINE_SOLVE, 1, launch_refine_solve2(Ds, Small{}, st, Sarr, D.B, D.nb_refine));
         return e;
@@ -331,7 +337,7 @@ struct GroupX : GroupBase {
         BBulkX<TW> Xs = X;
         Xs.e = const_cast<float2*>(v);
         Xs.lam2 = zlam;
-        RUN(1, launchbx_gradient<TW>(D, A, L, Xs, S, ff_tmp, st));
+        RUN(1, gradient(Xs, ff_tmp));
         RUN(1, launchbx_to_double(ff_tmp, out, (int64_t)D.n * D.B, st));
         return e;
     }
@@ -407,7 +413,7 @@ struct GroupX : GroupBase {
 
     cudaError_t step() override {
         cudaError_t e = cudaSuccess;
-        RUNC(BK_GRAD_APPEND, 1, launchbx_gradient<TW>(D, A, L, X, S, nullptr, st));
+        RUNC(BK_GRAD_APPEND, 1, gradient(X, nullptr));
         if (e == cudaSuccess) e = sketch_column();
         if (e == cudaSuccess) e = small_append();
         for (int r = 0; r < n_refine && e == cudaSuccess; ++r) e = refine();
@@ -464,21 +470,21 @@ struct GroupX : GroupBase {
             D.slice_kb = tune_pick(best, pick, t_def, def);
             D.nb_combine = batchx_combine_grid(D, sizeof(TW));
         }
-        if (T.ntiles) {   // instances per CTA of the tiled forward pass: the default or twice it
-            const int def_ic = sizeof(TW) == 4 ? 16 : 8;
+        if (T.ntiles && D.B >= kTileInst) {   // instances per CTA of the tiled forward pass: the default or half
             float best = 1e30f, t_def = 0.f;
             int pick = 0;
-            for (int ic : {0, 2 * def_ic}) {
+            for (int ic : {0, kTileInst / 2}) {
                 D.tile_ic = ic;
                 const float t = time_it([&] { return launchbx_tile_apply<TW>(D, T, X, S, part, st); });
-                log += " tile/" + std::to_string(ic ? ic : def_ic) + "=" + std::to_string(t);
+                log += " tile/" + std::to_string(tile_instances(D)) + "=" + std::to_string(t);
                 if (ic == 0) t_def = t;
                 if (t < best) { best = t; pick = ic; }
             }
             D.tile_ic = tune_pick(best, pick, t_def, 0);
         }
         if (A.kind == SGKS_OP_CSR) {
-            for (int which = T.ntiles ? 1 : 0; which < 2; ++which) {   // tiled: A w has no lanes to tune
+            for (int which = 0; which < 2; ++which) {
+                if (which == 0 ? T.ntiles : Tt.ntiles) continue;   // tiled passes have no lanes to tune
                 int* field = which == 0 ? &D.nl_a : &D.nl_t;
                 float best = 1e30f, t_def = 0.f;
                 int pick = *field;
@@ -503,8 +509,7 @@ struct GroupX : GroupBase {
         if (e != cudaSuccess) return e;
         tuned = "slice " + std::to_string(D.slice_kb) + " KB, lanes/row A " + std::to_string(D.nl_a) + ", A^T " +
                 std::to_string(D.nl_t) +
-                (T.ntiles ? ", tile instances " + std::to_string(D.tile_ic ? D.tile_ic : (sizeof(TW) == 4 ? 16 : 8))
-                          : std::string()) +
+                (T.ntiles ? ", tile instances " + std::to_string(tile_instances(D)) : std::string()) +
                 " (ms:" + log + ")";
         std::lock_guard<std::mutex> g(g_tune_mu);
         g_tune_cache[key] = TuneVal{D.slice_kb, D.nl_a, D.nl_t, D.tile_ic};
@@ -848,20 +853,27 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
     SketchLChunks LC{};   // S_L L w without storing L w
     rc = build_sketch_l_chunks(SK, L.p, s, kLChunk, LC, h->allocs, h->st, &why);
     if (rc != SGKS_OK) return bfail(h, rc, why);
-    // pixel tiles for the forward pass of a CSR operator on an image geometry (the regularizer's)
+    // pixel tiles of a CSR operator on an image geometry (the regularizer's)
     TiledA T{};
+    TiledT Tt{};
+    const std::vector<int> sizes = split_groups(inst.size(), max_group_size(o.ell + o.max_iters, o.n_refine, sizeof(float2)));
     if (op->kind == SGKS_OP_CSR && !(o.flags & SGKS_FLAG_NO_TILES) &&
         (reg->kind == SGKS_REG_GRAD2D || reg->kind == SGKS_REG_LAPLACE2D || reg->kind == SGKS_REG_SPACETIME)) {
         const int nt = reg->kind == SGKS_REG_SPACETIME ? reg->nt : 1;
-        rc = build_tiles(A.rp, A.ci, A.val, op->m, op->n, op->nnz, reg->nx, reg->ny, nt, 32, 16, T, h->allocs, h->st,
-                         &why);
+        // 32 x 16 pixels leave a third fewer partial sums than 16 x 16; below four CTAs per SM the
+        // smaller tile spreads the pass over the chip instead
+        const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, sizes[0] / kTileInst);
+        rc = build_tiles(A.rp, A.ci, A.val, op->m, op->n, op->nnz, reg->nx, reg->ny, nt, ctas < 4 * 152 ? 16 : 32, 16, T,
+                         h->allocs, h->st, &why);
+        if (rc == SGKS_OK)
+            rc = build_tiles_t(A.trp, A.tci, A.tval, op->m, op->n, op->nnz, reg->nx, reg->ny, nt, tile_ty(sizes[0]), tile_stage(sizes[0]), Tt, h->allocs, h->st, &why);
         if (rc != SGKS_OK) return bfail(h, rc, why);
     }
     const int dmax = o.ell + o.max_iters;
     if (o.n_refine > 0 && batch_refine_smem(dmax, 1, sizeof(float2)) > 200 * 1024)
         return bfail(h, SGKS_ERR_INVALID, "ell + max_iters too large for the batched refinement");
     size_t pos = 0;
-    for (const int B : split_groups(inst.size(), max_group_size(dmax, o.n_refine, sizeof(float2)))) {
+    for (const int B : sizes) {
         GroupX<TW>* G = new (std::nothrow) GroupX<TW>();
         if (!G) return bfail(h, SGKS_ERR_NOMEM, "host allocation failed");
         h->groups.push_back(G);
@@ -872,6 +884,7 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
         G->L = L;
         G->SK = SK;
         G->T = T;
+        G->Tt = Tt;
         G->LC = LC;
         G->io_dt = io_dt;
         G->has_xt = x_true != nullptr;
@@ -902,7 +915,7 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
         if (o.n_refine > 0) BA(X.r, nB);
         BA(lam2, B);
         BA(X.y2, (size_t)B * dmax);
-        if (T.ntiles) BA(G->part, (size_t)T.nseg * B);
+        if (T.ntiles) BA(G->part, (size_t)T.npart * B);
         // the FP64 setup of W_0 (Krylov basis, CGS2): its ell columns, a temporary and b
         BA(G->Xd.W, (size_t)D.ell * nB);
         BA(G->Xd.tm, mB);

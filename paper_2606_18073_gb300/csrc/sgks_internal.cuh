@@ -891,8 +891,7 @@ struct BDims {
     int nl_a, nl_t;           // CSR rows: lanes per row of A and of A^T (powers of two <= 32, tuned)
     int nb_refine;            // CTAs of kb_wtr (each leaves one partial per instance)
     int nb_setup;             // CTAs of the setup reductions
-    int tile_ic;              // tiled forward pass: instances per CTA (0: 16 for an FP32 basis, 8
-                              // for a float-float one; tuned)
+    int tile_ic;              // tiled forward pass: instances per CTA (0: kTileInst; tuned)
     int wait_tries;           // bounded waits of the bulk-copy combine's ring (kWaitTries; 0 in the
                               // timeout test of SGKS_TEST_TIMEOUT_GROUP, see sgks_batch.cu)
     double sketch_scale;      // 1/sqrt(zeta)
@@ -968,29 +967,61 @@ template <typename T>
 cudaError_t launchb_gather_in(const PtrPack& P, T* out, int64_t len, int B, cudaStream_t st);
 template <typename T>
 cudaError_t launchb_scatter_out(const T* in, const PtrPack& P, int64_t len, int B, cudaStream_t st);
-// A CSR operator re-blocked by pixel tiles for the batched forward pass (k_tiles.cu): the image
-// (nt frames of ny x nx) cut into TX x TY tiles; a segment is the run of one row's entries that
-// falls in one tile.  Segments are stored tile-major (the segments of tile t are
-// [tile_seg[t], tile_seg[t+1]), in row order), each with its entries (local pixel index within
-// the tile, value) and the slot of its partial sum; the slots of row r are
-// [ray_slot[r], ray_slot[r+1]), in the order of the row's entries.
+// A CSR operator re-blocked by pixel tiles for the batched passes (k_tiles.cu, k_tile_build.cu): the
+// image (nt frames of ny x nx) cut into TX x TY tiles.  Entries come in groups of four rows: pair k of
+// a group is four (slot, slot, value, value), one per row, at ent[4 (goff[g] + k)].
+// Forward: a segment is the run of one row's entries in one tile; the segments of tile t, longest
+// first, are the positions [4 tile_grp[t], 4 tile_grp[t+1]) (the last group filled up with empty ones);
+// row r's are ray_seg[ray_ptr[r] .. ray_ptr[r+1]), in the order of the row's entries.
 struct TiledA {
     int TX, TY, nx, ny, nt, ntx, nty, ntiles;
-    int64_t nseg;
-    const int32_t* tile_seg;   // [ntiles + 1]
-    const int32_t* seg_ent;    // [nseg + 1]
-    const int32_t* seg_slot;   // [nseg]
-    const int32_t* ray_slot;   // [m + 1]
-    const uint2* ent;          // [nnz] (local pixel index within the tile, value bits)
+    int64_t npart;             // segment positions: rows of the partial sums
+    const int32_t* order;      // tiles by descending work, so that the last CTAs are the short ones
+    const int32_t* tile_grp;   // [ntiles + 1]
+    const int32_t* goff;       // [npart / 4 + 1]
+    const int32_t* ray_ptr;    // [m + 1]
+    const int32_t* ray_seg;
+    const uint4* ent;          // slots: tile_slot of the pixel; TX TY holds 0
 };
-int build_tiles(const int32_t* d_rp, const int32_t* d_ci, const float* d_val, int64_t m, int64_t n, int64_t nnz,
-                int nx, int ny, int nt, int TX, int TY, TiledA& T, std::vector<void*>& allocs, cudaStream_t st,
-                std::string* why);
-size_t tile_smem(const TiledA& T, const BDims& D, size_t welem);
-// u_i = A w_i into column d_i of AW through the tiles (partials in part, nseg x B float-float)
+// Transposed: the rows of A that cross tile t are ray[tile_ray[t] .. tile_ray[t+1]), taken `stage` at a
+// time; stage tile_stage[t] + i has a group per four neighbouring pixels of the tile.
+struct TiledT {
+    int TX, TY, nx, ny, nt, ntx, nty, ntiles;   // ntiles = 0: not built
+    const int32_t* order;        // tiles by descending work
+    const int32_t* tile_stage;   // [ntiles + 1]
+    const int32_t* tile_ray;     // [ntiles + 1]
+    const int32_t* ray;
+    const int32_t* goff;         // [stages * TX TY / 4 + 1]
+    int stage;
+    const uint4* ent;            // slots: the row's place in its stage; `stage` holds 0
+};
+constexpr int kTileInst = 16;    // instances per CTA of the tiled passes
+constexpr int kTileAhead = 4;    // entry pairs behind the last group that may be read (and are not used)
+// rows of A staged at a time for a largest group of B instances: 64 KB of float-float values, 32 KB for
+// less than 8 (fewer stages, hence fewer barriers and less filling, while two CTAs still share an SM)
+inline int tile_stage(int B) { return B >= kTileInst ? 512 : (B >= 8 ? 1024 : (B >= 4 ? 1024 : (B >= 2 ? 2048 : 4096))); }
+// tiles of the transposed pass: 16 x 8 pixels for groups of 16 instances and more (a thread's
+// accumulators then leave registers for the loads: 2.4 -> 2.0 ms, 512^2 at 64), else 16 x 16
+constexpr int kTileTX = 16;
+inline int tile_ty(int B) { return B >= kTileInst ? 8 : 16; }
+// Shared-memory slot of local pixel q (row-major in a tile of width TX, TX even): neighbouring slots
+// swap on odd pixel rows.  With fewer than 128 bytes per pixel a load phase serves pixels of
+// neighbouring rays, which on rays along x lie one pixel row apart; the swap puts them in different
+// parts of a bank line, as pixels one column apart are.
+__host__ __device__ inline int tile_slot(int q, int TX) { return q ^ ((q / TX) & 1); }
+int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t m, int64_t n, int64_t nnz, int nx, int ny,
+                int nt, int TX, int TY, TiledA& T, std::vector<void*>& allocs, cudaStream_t st, std::string* why);
+int build_tiles_t(const int32_t* trp, const int32_t* tci, const float* tval, int64_t m, int64_t n, int64_t nnz, int nx,
+                  int ny, int nt, int TY, int stage, TiledT& T, std::vector<void*>& allocs, cudaStream_t st, std::string* why);
+int tile_instances(const BDims& D);   // instances per CTA of the forward pass
+// u_i = A w_i into column d_i of AW through the tiles (partials in part, npart x B float-float)
 template <typename TW>
 cudaError_t launchbx_tile_apply(const BDims& D, const TiledA& T, const BBulkX<TW>& X, const BSmall& S, float2* part,
                                 cudaStream_t st);
+// as launchbx_gradient
+template <typename TW>
+cudaError_t launchbx_tile_gradient(const BDims& D, const TiledT& T, const DevL& L, const BBulkX<TW>& X, const BSmall& S,
+                                   float2* out, cudaStream_t st);
 
 // compensated batched kernels (k_batchx.cu); TW = float or float2
 // a_rows = false: no A rows (they come from launchbx_tile_apply); l_rows = false: no t = L w
