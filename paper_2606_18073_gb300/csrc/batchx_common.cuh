@@ -1,5 +1,6 @@
 // Pieces shared by the compensated batched kernels (k_batchx.cu, k_tiles.cu): basis values in TW
-// (float or float2) into Dot2 accumulators, and the rows of L and L^T L in float-float.
+// (float or float2) into Dot2 accumulators, the rows of L and L^T L in float-float, and vectors staged in
+// shared memory row by row.
 #pragma once
 
 #include "batch_common.cuh"
@@ -166,5 +167,119 @@ struct StridedW {
     int64_t st;
     __device__ __forceinline__ TW operator()(int64_t q) const { return p[q * st]; }
 };
+
+// -------------------------------------------------- values staged in shared memory (k_tiles.cu, k_sketchx.cu)
+// Lane layout for IC staged instances: a lane takes VV of them (VV = 1: IC = 1, the halves of an
+// .f32x2 operand are then the two entries of a pair), G = IC / VV lanes per row.
+template <int IC>
+struct Lanes {
+    static constexpr int VV = IC >= 16 ? 4 : (IC >= 2 ? 2 : 1);
+    static constexpr int NP = VV == 4 ? 2 : 1;   // .f32x2 accumulators of a lane
+    static constexpr int G = IC / VV;
+    // Threads: two such pairs per lane take 80 registers, 256 threads then fill an SM three times over;
+    // with fewer instances a tile's CTA is small work and takes 512.
+    static constexpr int threads = IC >= 16 ? 256 : 512;
+};
+
+// A staged row in shared memory and a lane's part of it.
+template <typename TW, int IC>
+struct Staged;
+
+// float-float: pairs of instances as (hi0, hi1, lo0, lo1).  With 16 instances a row fills all banks; the
+// eight lanes of a load phase belong to two rows, and those of the odd one take the row's upper half
+// first, so that the phase touches every bank once.
+template <int IC>
+struct Staged<float2, IC> {
+    using LN = Lanes<IC>;
+    static constexpr int kRow = IC * 8;
+    int first;    // instance of accumulator 0
+    int second;   // of accumulator 1 (VV = 4)
+    const unsigned char *p0, *p1;
+    __device__ __forceinline__ Staged(const unsigned char* base, int j, int row) {
+        if constexpr (LN::VV == 4) {
+            const int c0 = j + ((row & 1) ? LN::G : 0), c1 = j + ((row & 1) ? 0 : LN::G);
+            first = 2 * c0;
+            second = 2 * c1;
+        } else {
+            first = second = LN::VV * j;
+        }
+        p0 = base + first * 8;
+        p1 = base + second * 8;
+    }
+    __device__ __forceinline__ int inst(int v) const { return (v < 2 ? first : second) + (v & 1); }
+    __device__ __forceinline__ void add(Dot2x2 (&d)[LN::NP], uint32_t slot, float c) const {
+        const f32x2 cc = pack2(c, c);
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p0 + slot * kRow);
+        d[0].add_prod2(cc, v.x, v.y);
+        if constexpr (LN::NP == 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(p1 + slot * kRow);
+            d[1].add_prod2(cc, w.x, w.y);
+        }
+    }
+    __device__ __forceinline__ void add_both(Dot2x2& d, uint32_t s0, uint32_t s1, float c0, float c1) const {
+        const float2 a = *reinterpret_cast<const float2*>(p0 + s0 * kRow), b = *reinterpret_cast<const float2*>(p0 + s1 * kRow);
+        d.add_prod2(pack2(c0, c1), pack2(a.x, b.x), pack2(a.y, b.y));
+    }
+    // values with the sign bits of m (0 or 0x80000000) turned over, exactly
+    static __device__ __forceinline__ f32x2 turned(f32x2 v, uint32_t m) { return v ^ (((f32x2)m << 32) | m); }
+    __device__ __forceinline__ void add_signed(Dot2x2 (&d)[LN::NP], uint32_t slot, uint32_t m) const {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p0 + slot * kRow);
+        d[0].accumulate(turned(v.x, m), turned(v.y, m));
+        if constexpr (LN::NP == 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(p1 + slot * kRow);
+            d[1].accumulate(turned(w.x, m), turned(w.y, m));
+        }
+    }
+    __device__ __forceinline__ void add_both_signed(Dot2x2& d, uint32_t s0, uint32_t s1, uint32_t m0, uint32_t m1) const {
+        const float2 a = *reinterpret_cast<const float2*>(p0 + s0 * kRow), b = *reinterpret_cast<const float2*>(p0 + s1 * kRow);
+        const f32x2 m = ((f32x2)m1 << 32) | m0;
+        d.accumulate(pack2(a.x, b.x) ^ m, pack2(a.y, b.y) ^ m);
+    }
+    // the lane's instances of row `slot`, v[k] instance inst(k)
+    __device__ __forceinline__ void put(unsigned char* base, int slot, const float2 (&v)[LN::VV]) const {
+        if constexpr (LN::VV == 1) {
+            *reinterpret_cast<float2*>(base + slot * kRow) = v[0];
+        } else {
+            *reinterpret_cast<float4*>(base + slot * kRow + first * 8) = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
+            if constexpr (LN::VV == 4)
+                *reinterpret_cast<float4*>(base + slot * kRow + second * 8) = make_float4(v[2].x, v[3].x, v[2].y, v[3].y);
+        }
+    }
+};
+
+// FP32 basis: plain values, a lane's VV next to each other
+template <int IC>
+struct Staged<float, IC> {
+    using LN = Lanes<IC>;
+    static constexpr int kRow = IC * 4;
+    int first;
+    const unsigned char* p0;
+    __device__ __forceinline__ Staged(const unsigned char* base, int j, int) : first(LN::VV * j), p0(base + LN::VV * j * 4) {}
+    __device__ __forceinline__ int inst(int v) const { return first + v; }
+    __device__ __forceinline__ void add(Dot2x2 (&d)[LN::NP], uint32_t slot, float c) const {
+        const f32x2 cc = pack2(c, c);
+        if constexpr (LN::NP == 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p0 + slot * kRow);
+            d[0].add_prod(cc, v.x);
+            d[1].add_prod(cc, v.y);
+        } else {
+            d[0].add_prod(cc, *reinterpret_cast<const f32x2*>(p0 + slot * kRow));
+        }
+    }
+    __device__ __forceinline__ void add_both(Dot2x2& d, uint32_t s0, uint32_t s1, float c0, float c1) const {
+        d.add_prod(pack2(c0, c1), pack2(*reinterpret_cast<const float*>(p0 + s0 * kRow), *reinterpret_cast<const float*>(p0 + s1 * kRow)));
+    }
+    __device__ __forceinline__ void put(unsigned char* base, int slot, const float (&v)[LN::VV]) const {
+#pragma unroll
+        for (int k = 0; k < LN::VV; ++k) *reinterpret_cast<float*>(base + slot * kRow + (first + k) * 4) = v[k];
+    }
+};
+
+// A batch of one: the sums of the first and of the second entries
+__device__ __forceinline__ Dot2 both_halves(const Dot2x2& a) {
+    Dot2 d = a.half(0);
+    d.merge(a.half(1));
+    return d;
+}
 
 }  // namespace sgks

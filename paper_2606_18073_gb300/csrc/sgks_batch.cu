@@ -293,15 +293,15 @@ struct GroupX : GroupBase {
     TiledA T{};                 // pixel tiles of a CSR A (ntiles = 0: the CSR-row kernel)
     TiledT Tt{};                // the same of A^T
     float2* part = nullptr;     // [npart][B] partial sums of the tiled forward pass
-    SketchLChunks LC{};         // S_L in column chunks of L w
-    float2* lpart = nullptr;    // [nchunks][s][B] partial sums of S_L L w
+    SketchChunks KC{};          // S_A and S_L in column chunks
+    float2* spart = nullptr;    // [nA + nL][s][B] partial sums of the sketches
 
     cudaError_t sketch_column() {
         cudaError_t e = cudaSuccess;
         if (T.ntiles) RUNC(BK_APPLY, 2, launchbx_tile_apply<TW>(D, T, X, S, part, st));
         else RUNC(BK_APPLY, 1, launchbx_apply_column<TW>(D, A, L, X, S, st, true, false));
-        RUNC(BK_SKETCH_L, 2, launchbx_sketch_l<TW>(D, L, X, LC, S, lpart, st));
-        RUNC(BK_GATHER, 1, launchbx_sketch_gather<TW>(D, X, SK, S, nullptr, nullptr, st, false));
+        RUNC(BK_SKETCH_L, 1, launchbx_sketch_chunks<TW>(D, L, X, KC, S, spart, st));
+        RUNC(BK_GATHER, 1, launchbx_sketch_reduce(D, KC, S, spart, st));
         return e;
     }
 
@@ -371,7 +371,7 @@ struct GroupX : GroupBase {
         if (e == cudaSuccess) e = cudaMemsetAsync(S.ka_done, 0, sizeof(int), st);
         RUN(1, launchbx_gather_in(bp, io_dt, X.b, D.m, B, st));
         RUN(1, launchbx_to_double(X.b, Xd.b, (int64_t)mB, st));
-        RUN(1, launchbx_sketch_gather<TW>(D, X, SK, S, X.b, S.Sb, st));
+        RUN(2, launchbx_sketch_vec<TW>(D, L, X, KC, S, X.b, spart, S.Sb, st));
         double* W = Xd.W;
         if (has_xt) {   // ||x_true||^2 from an FP64 copy (held in W_0's storage until W_0 is built)
             RUN(1, launchbx_gather_in(xtp, io_dt, X.xtrue, D.n, B, st));
@@ -850,13 +850,13 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
     rc = prepare_sparse_sign(sketch_key_host_dev(seed, 0), sketch_key_host_dev(seed, 1), op->m, L.p, s, o.zeta, SK,
                              h->allocs, h->d_err, h->st, &why);
     if (rc != SGKS_OK) return bfail(h, rc, why);
-    SketchLChunks LC{};   // S_L L w without storing L w
-    rc = build_sketch_l_chunks(SK, L.p, s, kLChunk, LC, h->allocs, h->st, &why);
-    if (rc != SGKS_OK) return bfail(h, rc, why);
     // pixel tiles of a CSR operator on an image geometry (the regularizer's)
     TiledA T{};
     TiledT Tt{};
     const std::vector<int> sizes = split_groups(inst.size(), max_group_size(o.ell + o.max_iters, o.n_refine, sizeof(float2)));
+    SketchChunks KC{};
+    rc = build_sketch_chunks(SK, op->m, L.p, s, sizes[0], KC, h->allocs, h->st, &why);
+    if (rc != SGKS_OK) return bfail(h, rc, why);
     if (op->kind == SGKS_OP_CSR && !(o.flags & SGKS_FLAG_NO_TILES) &&
         (reg->kind == SGKS_REG_GRAD2D || reg->kind == SGKS_REG_LAPLACE2D || reg->kind == SGKS_REG_SPACETIME)) {
         const int nt = reg->kind == SGKS_REG_SPACETIME ? reg->nt : 1;
@@ -885,7 +885,7 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
         G->SK = SK;
         G->T = T;
         G->Tt = Tt;
-        G->LC = LC;
+        G->KC = KC;
         G->io_dt = io_dt;
         G->has_xt = x_true != nullptr;
         for (int i = 0; i < B; ++i) {
@@ -911,7 +911,7 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
         BA(X.e, mB);
         BA(X.b, mB);
         if (G->has_xt) BA(X.xtrue, nB);
-        BA(G->lpart, (size_t)LC.nchunks * s * B);
+        BA(G->spart, (size_t)(KC.nA + KC.nL) * s * B);
         if (o.n_refine > 0) BA(X.r, nB);
         BA(lam2, B);
         BA(X.y2, (size_t)B * dmax);

@@ -727,13 +727,16 @@ struct DenseWork {
     int* cnt;
 };
 
-// S_L re-blocked by column chunks of t = L w (batched compensated forms): chunk c covers the
-// columns q in [c C, c C + C); the entries of sketch row r in chunk c are ent[seg[c s + r] ..
-// seg[c s + r + 1]), each (q - c C) | sign << 31, in the row's own order.  nchunks = 0: not built.
-struct SketchLChunks {
-    int C, nchunks;
-    const int32_t* seg;
-    const uint32_t* ent;
+// S_A and S_L re-blocked by chunks of C columns (batched compensated forms, k_sketchx.cu): nA chunks of
+// u = A w, then nL of t = L w.  The s sketch rows of a chunk, sorted by their number of entries, form
+// `groups` groups of four; group id = chunk groups + g holds the rows row[4 id ..] (-1: none) and the
+// quads goff[id] .. goff[id+1]: quad k is four entries (column in the chunk | sign << 31) of each of the
+// four rows, at ent[4 k + place in the group]; column C holds 0.
+struct SketchChunks {
+    int C, nA, nL, groups;
+    const int32_t* goff;
+    const int32_t* row;
+    const uint4* ent;
 };
 
 // ------------------------------------------------------------------------ launchers
@@ -1025,24 +1028,24 @@ cudaError_t launchbx_tile_gradient(const BDims& D, const TiledT& T, const DevL& 
 
 // compensated batched kernels (k_batchx.cu); TW = float or float2
 // a_rows = false: no A rows (they come from launchbx_tile_apply); l_rows = false: no t = L w
-// column (S_L L w comes from launchbx_sketch_l)
+// column (S_L L w comes from launchbx_sketch_chunks)
 template <typename TW>
 cudaError_t launchbx_apply_column(const BDims& D, const DevA<float, float>& A, const DevL& L, const BBulkX<TW>& X,
                                   const BSmall& S, cudaStream_t st, bool a_rows = true, bool l_rows = true);
-// l_rows = false: the S_A rows only
+// partial sums part[nA + nL][s][B] of S_A u_i and S_L L w_i for the newest column of every live instance
+// (L w is formed on the way, not stored), then their sums into S.partA and S.partL
 template <typename TW>
-cudaError_t launchbx_sketch_gather(const BDims& D, const BBulkX<TW>& X, const SketchCSR& SK, const BSmall& S,
-                                   const float2* vec, double* out_vec, cudaStream_t st, bool l_rows = true);
-// S_L L w_i for the newest column of every live instance through the column chunks of S_L, without
-// storing L w: part[nchunks][s][B] per-chunk partial sums, then S.partL.
+cudaError_t launchbx_sketch_chunks(const BDims& D, const DevL& L, const BBulkX<TW>& X, const SketchChunks& K,
+                                   const BSmall& S, float2* part, cudaStream_t st);
+cudaError_t launchbx_sketch_reduce(const BDims& D, const SketchChunks& K, const BSmall& S, const float2* part,
+                                   cudaStream_t st);
+// S_A v_i, scaled, for an m-vector v [m][B], to out [B][s] (at the setup, while S.sc is zero)
 template <typename TW>
-cudaError_t launchbx_sketch_l(const BDims& D, const DevL& L, const BBulkX<TW>& X, const SketchLChunks& LC,
-                              const BSmall& S, float2* part, cudaStream_t st);
-// column chunks of S_L (device arrays to allocs); chunk length C
-int build_sketch_l_chunks(const SketchCSR& SK, int64_t p, int s, int C, SketchLChunks& LC,
-                          std::vector<void*>& allocs, cudaStream_t st, std::string* why);
-size_t sketch_l_smem(int B);
-constexpr int kLChunk = 2048;   // columns of L w per chunk of S_L
+cudaError_t launchbx_sketch_vec(const BDims& D, const DevL& L, const BBulkX<TW>& X, const SketchChunks& K,
+                                const BSmall& S, const float2* vec, float2* part, double* out, cudaStream_t st);
+// chunks for a largest group of B instances (device arrays to allocs)
+int build_sketch_chunks(const SketchCSR& SK, int64_t m, int64_t p, int s, int B, SketchChunks& K,
+                        std::vector<void*>& allocs, cudaStream_t st, std::string* why);
 template <typename TW>
 cudaError_t launchbx_combine(const BDims& D, const BBulkX<TW>& X, const BSmall& S, int mode, cudaStream_t st);
 template <typename TW>
