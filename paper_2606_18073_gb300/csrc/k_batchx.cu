@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kThreads) kbx_apply_column(BDims D, DevA<float
 
 // ------------------------------------------------------------------- a5 + a6: combine
 // x_i = W_i y_i and e_i = (A W_i) y_i - b_i with Dot2, y_i as float-float pairs laid out [j][B]
-// (kbx_split_y).  The items of a CTA are (tile, column) pairs: one SB-byte slice of one column
+// (written with y, k_small2.cu).  The items of a CTA are (tile, column) pairs: one SB-byte slice of one column
 // of W (x tiles, SB / sizeof(TW) values) or of A W (e tiles, SB / 8 values), streamed through an
 // NS-stage ring filled by cp.async.bulk.  Stage s has two mbarriers: full[s] (the copy landed)
 // and empty[s] (every consumer warp has read it; one arrival per warp).  kCombConsumers threads
@@ -573,6 +573,7 @@ __global__ void __launch_bounds__(kThreads) kbx_gradient(BDims D, DevA<float, fl
 // lane sums go to FP64 in shared memory, one partial per CTA and instance.
 template <typename TW, int NB>
 __global__ void __launch_bounds__(kThreads, 2) kbx_wtr(BDims D, BBulkX<TW> X, BSmall S, const float2* __restrict__ r) {
+    pdl_trigger();   // the refinement solve loads X meanwhile
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_dlive;
     __shared__ int s_stop[kMaxBatch];
@@ -629,16 +630,6 @@ __global__ void __launch_bounds__(kThreads, 2) kbx_wtr(BDims D, BBulkX<TW> X, BS
 }
 
 // ------------------------------------------------------------------------ conversions
-// y_i (FP64 from the small phase, y[i * dmax + j]) split into float-float once per combine and
-// transposed to y2[j * B + i], so that the B threads of one column read consecutive pairs
-__global__ void kbx_split_y(const double* __restrict__ y, float2* __restrict__ y2, int B, int dmax) {
-    const int len = B * dmax;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < len; t += gridDim.x * blockDim.x) {
-        const int j = t / B, i = t - j * B;
-        y2[t] = dsplit(y[(size_t)i * dmax + j]);
-    }
-}
-
 __global__ void kbx_gather_in(PtrPack P, int in_dt, float2* __restrict__ out, int64_t len, int B) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < len * B; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t q = t / B;
@@ -749,10 +740,6 @@ int batchx_combine_grid(const BDims& D, size_t welem) {
 
 template <typename TW>
 cudaError_t launchbx_combine(const BDims& D, const BBulkX<TW>& X, const BSmall& S, int mode, cudaStream_t st) {
-    const int ylen = D.B * D.dmax;
-    kbx_split_y<<<(ylen + kThreads - 1) / kThreads, kThreads, 0, st>>>(S.y, X.y2, D.B, D.dmax);
-    cudaError_t e0 = cudaGetLastError();
-    if (e0 != cudaSuccess) return e0;
     if (D.tma) {
         const size_t smem = batchx_combine_smem(sizeof(TW), D.slice_kb);
         auto k = D.slice_kb == 8 ? kbx_combine_tma<TW, 6, 8192> : kbx_combine_tma<TW, 4, 16384>;

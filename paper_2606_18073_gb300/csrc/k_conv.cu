@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_column_conv(Dims D, DevA<T, 
 template <typename T, typename V, int MODE, int K, int CB>
 __global__ void __launch_bounds__(kThreads) k_gradient_refine2(Dims D, DevA<T, V> A, DevL L, Bulk<T> B, Small S) {
     pdl_wait();   // all global reads below depend on the previous kernel
+    pdl_trigger();   // the refinement solve loads X meanwhile
     using VT = typename Vec16<T>::type;
     constexpr int NPV = 16 / (int)sizeof(T);              // values per 16-byte vector
     constexpr int NV = kThreads / NPV / 32;                 // vectors per lane per column of a tile

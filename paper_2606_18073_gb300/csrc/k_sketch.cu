@@ -114,6 +114,7 @@ template <typename TA, typename TL, typename Acc>
 __global__ void __launch_bounds__(kThreads) k_sketch_gather_col(Dims D, const TA* __restrict__ AW, const TL* __restrict__ lw,
                                                                 SketchCSR SK, Small S) {
     pdl_wait();   // all global reads below depend on the previous kernel
+    pdl_trigger();   // the QR append loads its earlier columns meanwhile
     __shared__ double red[kWarps];
     const DevScalars* sc = S.sc;
     if (sc->stop) return;

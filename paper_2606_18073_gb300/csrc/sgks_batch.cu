@@ -319,7 +319,7 @@ struct GroupX : GroupBase {
 
     cudaError_t refine() {
         cudaError_t e = cudaSuccess;
-        RUNC(BK_COMBINE_REFINE, 2, launchbx_combine<TW>(D, X, S, 0, st));
+        RUNC(BK_COMBINE_REFINE, 1, launchbx_combine<TW>(D, X, S, 0, st));
         RUNC(BK_GRAD_REFINE, 1, gradient(X, X.r));
         RUNC(BK_GRAD_REFINE, 1, launchbx_wtr<TW>(D, X, S, X.r, st));
         RUNC(BK_REFINE_SOLVE, 1, launch_refine_solve2(Ds, Small{}, st, Sarr, D.B, D.nb_refine));
@@ -407,7 +407,7 @@ struct GroupX : GroupBase {
             if (e == cudaSuccess) e = small_append();
         }
         for (int r = 0; r < n_refine && e == cudaSuccess; ++r) e = refine();
-        RUN(2, launchbx_combine<TW>(D, X, S, 2, st));
+        RUN(1, launchbx_combine<TW>(D, X, S, 2, st));
         return e;
     }
 
@@ -417,7 +417,7 @@ struct GroupX : GroupBase {
         if (e == cudaSuccess) e = sketch_column();
         if (e == cudaSuccess) e = small_append();
         for (int r = 0; r < n_refine && e == cudaSuccess; ++r) e = refine();
-        RUNC(BK_COMBINE, 2, launchbx_combine<TW>(D, X, S, 1, st));
+        RUNC(BK_COMBINE, 1, launchbx_combine<TW>(D, X, S, 1, st));
         return e;
     }
 
@@ -614,7 +614,7 @@ int max_group_size(int dmax, int n_refine, size_t elem) {
 // value, velem: bytes of the other vectors' values; comb_grid(D): CTAs of the group's combine.
 template <typename CG>
 int init_group(sgks_batch* h, GroupBase* G, const sgks_op* op, const DevL& L, int B, int s, const sgks_options& o,
-               int cluster2, size_t welem, size_t velem, const double* lambdas, CG&& comb_grid) {
+               int cluster2, size_t welem, size_t velem, const double* lambdas, CG&& comb_grid, float2** y2 = nullptr) {
     const int dmax = o.ell + o.max_iters;
     G->nnz = op->kind == SGKS_OP_CSR ? op->nnz : 0;
     G->n_refine = o.n_refine;
@@ -709,6 +709,7 @@ int init_group(sgks_batch* h, GroupBase* G, const sgks_op* op, const DevL& L, in
     BA(Tm, B * dm2);
     BA(dA, (size_t)B * dmax);
     BA(G->Sarr, B);
+    if (y2) BA(*y2, (size_t)B * dmax);
 #undef BA
     if (e != cudaSuccess) return bfail(h, SGKS_ERR_NOMEM, std::string("device allocation: ") + cudaGetErrorString(e));
     std::vector<Small> sm((size_t)B);
@@ -734,6 +735,8 @@ int init_group(sgks_batch* h, GroupBase* G, const sgks_op* op, const DevL& L, in
         q.gpart = S.gpart + (size_t)i * D.nb_refine * dmax;
         q.sc = S.sc + i;
         q.lam = lambdas[G->members[i]];
+        q.y2 = y2 ? *y2 + i : nullptr;
+        q.y2_stride = B;
         lam[i] = q.lam;
     }
     e = cudaMemcpy(G->Sarr, sm.data(), sizeof(Small) * B, cudaMemcpyHostToDevice);
@@ -893,7 +896,7 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
             G->xtp.p[i] = x_true ? x_true[G->members[i]] : nullptr;
         }
         rc = init_group(h, G, op, L, B, s, o, cluster2, sizeof(TW), sizeof(float2), lambdas,
-                        [](const BDims& D) { return batchx_combine_grid(D, sizeof(TW)); });
+                        [](const BDims& D) { return batchx_combine_grid(D, sizeof(TW)); }, &G->X.y2);
         if (rc != SGKS_OK) return rc;
         const BDims& D = G->D;
         cudaError_t e = cudaSuccess;
@@ -914,7 +917,6 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
         BA(G->spart, (size_t)(KC.nA + KC.nL) * s * B);
         if (o.n_refine > 0) BA(X.r, nB);
         BA(lam2, B);
-        BA(X.y2, (size_t)B * dmax);
         if (T.ntiles) BA(G->part, (size_t)T.npart * B);
         // the FP64 setup of W_0 (Krylov basis, CGS2): its ell columns, a temporary and b
         BA(G->Xd.W, (size_t)D.ell * nB);
