@@ -84,10 +84,8 @@ __global__ void __launch_bounds__(kThreads) kd_dot_acc(const double* __restrict_
 
 // acc += sign * sum_b part[b]  (the CTA partials of a dot product, in order)
 __global__ void kd_acc_parts(const double* __restrict__ part, int nb, double sign, double* acc) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double v = 0.0;
-    for (int b = 0; b < nb; ++b) v += part[b];
-    *acc += sign * v;
+    const double v = warp_sum_parts(part, nb);   // one warp
+    if (lane_id() == 0) *acc += sign * v;
 }
 
 // out[j] = scale * sum_k sign_k u[row_k] over the zeta entries of column j of the sparse-sign

@@ -22,26 +22,6 @@ __device__ __forceinline__ double dense_val(double v) { return v; }
 __device__ __forceinline__ double dense_val(float v) { return (double)v; }
 __device__ __forceinline__ double dense_val(float2 v) { return (double)v.x + (double)v.y; }
 
-// Sums over the warp of R values per lane: at each step half of the lanes take over half of the
-// values, until a lane holds one row's sum; lane & (32 / R - 1) == 0 then holds row lane / (32 / R).
-template <int R>
-__device__ __forceinline__ double warp_sum_rows(double (&a)[R]) {
-    const int lane = lane_id();
-    int off = 16;
-#pragma unroll
-    for (int h = R / 2; h >= 1; h >>= 1, off >>= 1) {
-        const bool up = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const double keep = up ? a[i + h] : a[i], send = up ? a[i] : a[i + h];
-            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-    }
-    double v = a[0];
-    for (; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
-
 // Rows [g R, g R + R) of SG (s x len) times v over the columns [c C, c C + C); nc chunks a row.
 template <int R, typename TV>
 __device__ void dense_rows(const double* __restrict__ SG, const TV* __restrict__ v, int64_t len, int s, int64_t C, int nc,

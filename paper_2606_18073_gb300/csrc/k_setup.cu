@@ -133,10 +133,27 @@ cudaError_t launch_apply(const Dims& D, const DevA<T, V>& A, const DevL& L, int 
 }
 
 // ------------------------------------------------------------------------ n-vector algebra
-// part[b*k + c] = sum over the rows of CTA b of V0[c][i] * w[i]
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_dots(const T* __restrict__ V0, int64_t n, int k, const T* __restrict__ w,
-                                                   double* part) {
+// part[b*k + c] = sum over the rows of CTA b of V0[c][i] * w[i]: the CTA's rows of w staged in shared
+// memory, two columns per warp (tile_dots)
+__global__ void __launch_bounds__(kThreads) k_dots(const double* __restrict__ V0, int64_t n, int k,
+                                                   const double* __restrict__ w, double* part) {
+    extern __shared__ double acc[];   // [k]
+    __shared__ double us[kThreads];
+    for (int c = threadIdx.x; c < k; c += kThreads) acc[c] = 0.0;
+    for (int64_t i0 = (int64_t)blockIdx.x * kThreads; i0 < n; i0 += (int64_t)gridDim.x * kThreads) {
+        const int rows = (int)min((int64_t)kThreads, n - i0);
+        __syncthreads();
+        if (threadIdx.x < rows) us[threadIdx.x] = w[i0 + threadIdx.x];
+        __syncthreads();
+        tile_dots<double>(V0 + i0, (size_t)n, us, rows, k, acc);
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < k; c += kThreads) part[(size_t)blockIdx.x * k + c] = acc[c];
+}
+
+// the same for FP32 vectors, products in FP64
+__global__ void __launch_bounds__(kThreads) k_dots_f32(const float* __restrict__ V0, int64_t n, int k,
+                                                       const float* __restrict__ w, double* part) {
     __shared__ double red[kWarps];
     for (int c = 0; c < k; ++c) {
         double a = 0.0;
@@ -145,11 +162,7 @@ __global__ void __launch_bounds__(kThreads) k_dots(const T* __restrict__ V0, int
         a = warp_sum(a);
         if (lane_id() == 0) red[warp_id()] = a;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int q = 0; q < kWarps; ++q) t += red[q];
-            part[(size_t)blockIdx.x * k + c] = t;
-        }
+        if (threadIdx.x == 0) part[(size_t)blockIdx.x * k + c] = tree_sumd<kWarps>(red);
         __syncthreads();
     }
 }
@@ -159,10 +172,9 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads) k_orth_update(T* w, const T* __restrict__ V0, int64_t n, int k,
                                                           const double* __restrict__ part, int nb) {
     __shared__ double coef[8];
-    if (threadIdx.x < k) {
-        double t = 0.0;
-        for (int b = 0; b < nb; ++b) t += part[(size_t)b * k + threadIdx.x];
-        coef[threadIdx.x] = t;
+    if (warp_id() < k) {   // k < kWarps: a warp per coefficient
+        const double t = warp_sum_parts(part + warp_id(), nb, k);
+        if (lane_id() == 0) coef[warp_id()] = t;
     }
     __syncthreads();
     for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) {
@@ -175,20 +187,27 @@ __global__ void __launch_bounds__(kThreads) k_orth_update(T* w, const T* __restr
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_normalize(T* w, int64_t n, const double* __restrict__ part, int nb) {
     __shared__ double inv;
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int b = 0; b < nb; ++b) t += part[b];
-        inv = 1.0 / sqrt(t);
+    if (warp_id() == 0) {
+        const double t = warp_sum_parts(part, nb);
+        if (lane_id() == 0) inv = 1.0 / sqrt(t);
     }
     __syncthreads();
     for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads)
         w[i] = (T)((double)w[i] * inv);
 }
 
+static void dots_go(const double* V0, int64_t n, int k, const double* w, double* part, int nb, cudaStream_t st) {
+    carveout_once((const void*)k_dots);
+    k_dots<<<nb, kThreads, sizeof(double) * (size_t)k, st>>>(V0, n, k, w, part);
+}
+static void dots_go(const float* V0, int64_t n, int k, const float* w, double* part, int nb, cudaStream_t st) {
+    carveout_once((const void*)k_dots_f32);
+    k_dots_f32<<<nb, kThreads, 0, st>>>(V0, n, k, w, part);
+}
+
 template <typename T>
 cudaError_t launch_dots(const T* V0, int64_t n, int k, const T* w, double* part, int nb, cudaStream_t st) {
-    carveout_once((const void*)k_dots<T>);
-    k_dots<T><<<nb, kThreads, 0, st>>>(V0, n, k, w, part);
+    dots_go(V0, n, k, w, part, nb, st);
     return cudaGetLastError();
 }
 template <typename T>
@@ -199,8 +218,7 @@ cudaError_t launch_orth_update(T* w, const T* V0, int64_t n, int k, const double
 }
 template <typename T>
 cudaError_t launch_sqnorm(const T* w, int64_t n, double* part, int nb, cudaStream_t st) {
-    carveout_once((const void*)k_dots<T>);
-    k_dots<T><<<nb, kThreads, 0, st>>>(w, n, 1, w, part);
+    dots_go(w, n, 1, w, part, nb, st);
     return cudaGetLastError();
 }
 template <typename T>

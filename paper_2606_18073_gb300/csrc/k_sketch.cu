@@ -213,18 +213,25 @@ cudaError_t launch_gaussian_sketch(const Dims& D, const DevA<T, V>& A, const Dev
     return launch_dense_pair<T, T>(D, B.AW, B.tmp_p, S, SA, SL, K, st);
 }
 
-// out[i] = scale * sum_{b < nb} part[b*len + i], summed in b order.
-__global__ void k_reduce_rows(const double* __restrict__ part, int nb, int len, double scale, double* out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// out[i] = scale * sum_{b < nb} part[b*len + i]: a warp per sum, lanes over the partials
+__global__ void __launch_bounds__(kThreads) k_reduce_rows(const double* __restrict__ part, int nb, int len, double scale,
+                                                          double* out) {
+    const int i = blockIdx.x * kWarps + warp_id();
     if (i >= len) return;
-    double v = 0.0;
-    for (int b = 0; b < nb; ++b) v += part[(size_t)b * len + i];
-    out[i] = scale * v;
+    const double v = warp_sum_parts(part + i, nb, len);
+    if (lane_id() == 0) out[i] = scale * v;
+}
+
+// the same for one partial each
+__global__ void k_scale_rows(const double* __restrict__ part, int len, double scale, double* out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < len) out[i] = scale * part[i];
 }
 
 cudaError_t launch_reduce_rows(const double* part, int nb, int len, double scale, double* out, cudaStream_t st) {
     carveout_once((const void*)k_reduce_rows);
-    k_reduce_rows<<<(len + kThreads - 1) / kThreads, kThreads, 0, st>>>(part, nb, len, scale, out);
+    if (nb == 1) k_scale_rows<<<(len + kThreads - 1) / kThreads, kThreads, 0, st>>>(part, len, scale, out);
+    else k_reduce_rows<<<(len + kWarps - 1) / kWarps, kThreads, 0, st>>>(part, nb, len, scale, out);
     return cudaGetLastError();
 }
 

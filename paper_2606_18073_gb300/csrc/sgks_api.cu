@@ -15,7 +15,6 @@
 #include <stdio.h>
 
 #include <atomic>
-#include <type_traits>
 #include <new>
 #include <algorithm>
 #include <string>
@@ -581,48 +580,51 @@ struct EngineGKS : Engine<T, V> {
     using Base::D; using Base::S; using Base::A; using Base::L; using Base::B; using Base::st;
     using Base::host_d; using Base::timed; using Base::b_own;
     T *QA = nullptr, *QL = nullptr;        // [dmax][m], [dmax][p]
-    double *gpart = nullptr, *vpart = nullptr;
-    double *c1 = nullptr, *c2 = nullptr;   // projection coefficients [dmax]
-    double* sc4 = nullptr;                 // n0, n1, scale, spare
+    double *gpart = nullptr, *vpart = nullptr;   // of both factors, one behind the other
+    double *c1 = nullptr, *c2 = nullptr;   // projection coefficients [2][dmax + 1]
+    double* sc4 = nullptr;                 // scale of the basis column and of the two factors'
     int* flag = nullptr;
     double tau = 1e-10;                    // eq. loss_criterion
-
-    cudaError_t qr_col(T* Q, int64_t h, double* Rm, double* out, bool with_b) {
-        const DevScalars* sc = S.sc;
-        const int dm = D.dmax;
-        cudaError_t e = cudaSuccess;
-        auto R = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-        R(launchg_dot<T>(Q, h, nullptr, sc, vpart, sc4 + 0, st));
-        for (int pass = 0; pass < 2; ++pass) {
-            double* c = pass ? c2 : c1;
-            R(launchg_coef<T>(Q, h, Q, sc, dm, gpart, c, st));
-            R(launchg_update<T>(Q, h, sc, c, nullptr, dm, st));
-        }
-        R(launchg_dot<T>(Q, h, nullptr, sc, vpart, sc4 + 1, st));
-        R(launchg_qr_finish(c1, c2, sc, dm, sc4 + 0, sc4 + 1, Rm, out, sc4 + 2, st));
-        R(launchg_scale<T>(Q, h, sc, sc4 + 2, st));
-        if (with_b) R(launchg_dot<T>(Q, h, b_own, sc, vpart, out + 3, st));
-        g_launches.fetch_add(2 + 4 * 2 + 2 + 1 + 1 + (with_b ? 2 : 0));
-        return e;
-    }
 
     // column d of V (= W) against V[:, :d]: CGS, a second pass when ||V^T v|| >= tau ||v||, normalise
     cudaError_t orth_new() {
         const DevScalars* sc = S.sc;
         const int dm = D.dmax;
-        T* Vm = B.W;
+        GJobs<T> J{};
+        J.n = 1;
+        J.j[0] = GJob<T>{B.W, D.n, nullptr, 0, nullptr, gpart, vpart, c1, c2, nullptr, nullptr, sc4};
         cudaError_t e = cudaSuccess;
         auto R = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-        R(launchg_coef<T>(Vm, D.n, Vm, sc, dm, gpart, c1, st));
-        R(launchg_update<T>(Vm, D.n, sc, c1, nullptr, dm, st));
-        R(launchg_coef<T>(Vm, D.n, Vm, sc, dm, gpart, c2, st));
-        R(launchg_dot<T>(Vm, D.n, nullptr, sc, vpart, sc4 + 1, st));
-        R(launchg_loss(c2, sc, sc4 + 1, tau, flag, st));
-        R(launchg_update<T>(Vm, D.n, sc, c2, flag, dm, st));
-        R(launchg_dot<T>(Vm, D.n, nullptr, sc, vpart, sc4 + 1, st));
-        R(launchg_inv_norm(sc4 + 1, sc4 + 2, S.sc, st));
-        R(launchg_scale<T>(Vm, D.n, sc, sc4 + 2, st));
-        g_launches.fetch_add(2 + 1 + 2 + 2 + 1 + 1 + 2 + 1 + 1);
+        R(launchg_coef<T>(J, sc, dm, 0, st));
+        R(launchg_update<T>(J, sc, dm, 0, nullptr, st));
+        R(launchg_coef<T>(J, sc, dm, 1, st));
+        R(launchg_loss(c2, sc, tau, flag, st));
+        R(launchg_update<T>(J, sc, dm, 1, flag, st));
+        R(launchg_inv_norm(vpart, gks_vec_blocks(D.n), sc4, S.sc, st));
+        R(launchg_scale<T>(J, sc, st));
+        g_launches.fetch_add(2 + 1 + 2 + 1 + 1 + 1 + 1);
+        return e;
+    }
+
+    // A v (column d of A V) and L v appended to Q_A and Q_L by two projections each, both factors in the
+    // same launches: R columns, the flags and the d_A entry in S.qr_out
+    cudaError_t qr_cols() {
+        const DevScalars* sc = S.sc;
+        const int dm = D.dmax;
+        GJobs<T> J{};
+        J.n = 2;
+        J.j[0] = GJob<T>{QA, D.m, B.AW, 1, b_own, gpart, vpart, c1, c2, S.RA, S.qr_out, sc4 + 1};
+        J.j[1] = GJob<T>{QL, D.p, B.tmp_p, 0, nullptr, gpart + (size_t)gks_blocks(D.m) * (dm + 1),
+                         vpart + 2 * (size_t)gks_vec_blocks(D.m), c1 + dm + 1, c2 + dm + 1, S.RL, S.qr_out + 4, sc4 + 2};
+        cudaError_t e = cudaSuccess;
+        auto R = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
+        for (int pass = 0; pass < 2; ++pass) {
+            R(launchg_coef<T>(J, sc, dm, pass, st));
+            R(launchg_update<T>(J, sc, dm, pass, nullptr, st));
+        }
+        R(launchg_qr_finish<T>(J, sc, dm, st));
+        R(launchg_scale<T>(J, sc, st));
+        g_launches.fetch_add(2 * 3 + 2);
         return e;
     }
 
@@ -631,14 +633,7 @@ struct EngineGKS : Engine<T, V> {
         cudaError_t e = cudaSuccess;
         auto R = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
         R(timed(PK_SKETCH, d, [&] { return launch_apply_new_column<T, V>(D, A, L, B, S, st); }));
-        R(launchg_copy_col<T>(B.AW, QA, D.m, S.sc, true, st));      // A v (column d of A V)
-        R(launchg_copy_col<T>(B.tmp_p, QL, D.p, S.sc, false, st));  // L v (a p-vector)
-        g_launches.fetch_add(2);
-        R(timed(PK_QR_APPEND, d, [&] {
-            cudaError_t e2 = qr_col(QA, D.m, S.RA, S.qr_out, true);
-            if (e2 == cudaSuccess) e2 = qr_col(QL, D.p, S.RL, S.qr_out + 4, false);
-            return e2;
-        }));
+        R(timed(PK_QR_APPEND, d, [&] { return qr_cols(); }));
         R(timed(PK_STACKED_SOLVE, d, [&] { return launch_stacked_solve(D, S, st); }));
         return e;
     }
@@ -1181,10 +1176,10 @@ static int build_engine(sgks_handle* h, const sgks_op* op, const sgks_reg* reg, 
         const int64_t hmax = std::max<int64_t>(std::max<int64_t>(D.n, D.m), D.p);
         AL(EG->QA, dm * D.m);
         AL(EG->QL, dm * D.p);
-        AL(EG->gpart, (size_t)gks_blocks(hmax) * dm);
-        AL(EG->vpart, (size_t)gks_vec_blocks(hmax));
-        AL(EG->c1, dm);
-        AL(EG->c2, dm);
+        AL(EG->gpart, (size_t)(gks_blocks(hmax) + gks_blocks(D.m) + gks_blocks(D.p)) * (dm + 1));
+        AL(EG->vpart, 2 * (size_t)(gks_vec_blocks(hmax) + gks_vec_blocks(D.m) + gks_vec_blocks(D.p)));
+        AL(EG->c1, 2 * (dm + 1));
+        AL(EG->c2, 2 * (dm + 1));
         AL(EG->sc4, 4);
         AL(EG->flag, 1);
     }

@@ -203,6 +203,55 @@ __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 template <typename T>
 __device__ __forceinline__ double warp_sum_acc(T v) { return (double)warp_sum(v); }
 
+// Sums over the warp of R values per lane: at each step half of the lanes take over half of the
+// values, until a lane holds one row's sum; lane & (32 / R - 1) == 0 then holds row lane / (32 / R).
+template <int R>
+__device__ __forceinline__ double warp_sum_rows(double (&a)[R]) {
+    const int lane = lane_id();
+    int off = 16;
+#pragma unroll
+    for (int h = R / 2; h >= 1; h >>= 1, off >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double keep = up ? a[i + h] : a[i], send = up ? a[i] : a[i + h];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+    double v = a[0];
+    for (; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+}
+
+// Sum of part[0 .. nb) over the calling warp (lanes over the entries), in every lane.
+__device__ __forceinline__ double warp_sum_parts(const double* part, int nb, int stride = 1) {
+    double a = 0.0;
+#pragma unroll 4
+    for (int b = lane_id(); b < nb; b += 32) a += __ldcg(part + (size_t)b * stride);
+    return warp_sum(a);
+}
+
+// acc[j] += sum over q < rows of Q[j ld + q] us[q], j < d: two columns per warp and step, lanes over the
+// rows, products in T; the two sums share their reduction (an FP64 warp instruction takes a quarter of the
+// SM for 64 clocks).  us and acc in shared memory, acc[j] owned by the warp that takes column j.
+template <typename T>
+__device__ __forceinline__ void tile_dots(const T* __restrict__ Q, size_t ld, const T* us, int rows, int d, double* acc) {
+    for (int j = 2 * warp_id(); j < d; j += 2 * kWarps) {
+        const T *q0 = Q + (size_t)j * ld, *q1 = j + 1 < d ? q0 + ld : q0;
+        T a0 = T(0), a1 = T(0);
+#pragma unroll 4
+        for (int q = lane_id(); q < rows; q += 32) {
+            const T u = us[q];
+            a0 += q0[q] * u;
+            a1 += q1[q] * u;
+        }
+        double s[2] = {(double)a0, (double)a1};
+        const double v = warp_sum_rows<2>(s);
+        const int c = j + (lane_id() >> 4);
+        if ((lane_id() & 15) == 0 && c < d) acc[c] += v;
+    }
+}
+
 // Fixed pairwise tree over N values with a stride (deterministic, log2 depth).
 template <int N>
 __device__ __forceinline__ double tree_sumd(const double* a, int stride = 1) {
@@ -1072,26 +1121,43 @@ cudaError_t launchd_kbar(const T* Wb0, int64_t n, int ell, const double* Rinv, T
 template <typename T, typename V>
 cudaError_t launch_apply_new_column(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B,
                                     const Small& S, cudaStream_t st);
+// One factor that a column is appended to or projected against: column d of Q (h rows), its coefficients.
+template <typename T>
+struct GJob {
+    T* Q;                // [.][h]
+    int64_t h;
+    const T* src;        // the new column is copied from here first (+ d h when src_col); null: it is in Q
+    int src_col;
+    const T* b;          // the partials of the updated column's product with b are wanted; or null
+    double* part;        // [gks_blocks(h)][dm + 1]: products with the columns before it, squared norm
+    double* npart;       // [gks_vec_blocks(h)][2]: squared norm and product with b after an update
+    double *c1, *c2;     // [dm + 1] sums of part in the first and the second pass
+    double* Rm;          // R, column d is written
+    double* out;         // rho, breakdown, finite, d_A entry (layout of S.qr_out)
+    double* scale;       // 1 / norm of the new column
+};
+template <typename T>
+struct GJobs {
+    GJob<T> j[2];
+    int n;
+};
 int gks_blocks(int64_t h);
 int gks_vec_blocks(int64_t h);
+// pass 0: copy the new column (src), part; then c1.  pass 1: part, then c2.
 template <typename T>
-cudaError_t launchg_coef(const T* Q, int64_t h, const T* U, const DevScalars* sc, int dm, double* part, double* c,
-                         cudaStream_t st);
+cudaError_t launchg_coef(const GJobs<T>& J, const DevScalars* sc, int dm, int pass, cudaStream_t st);
+// column d -= Q[:, :d] c (c1 for pass 0, c2 for pass 1; skipped when flag is given and 0); npart for pass 1
 template <typename T>
-cudaError_t launchg_update(T* Q, int64_t h, const DevScalars* sc, const double* c, const int* flag, int dm,
-                           cudaStream_t st);
+cudaError_t launchg_update(const GJobs<T>& J, const DevScalars* sc, int dm, int pass, const int* flag, cudaStream_t st);
+// column d of R, out and scale from c1, c2 and npart
 template <typename T>
-cudaError_t launchg_dot(const T* U, int64_t h, const T* w, const DevScalars* sc, double* part, double* out,
-                        cudaStream_t st);
+cudaError_t launchg_qr_finish(const GJobs<T>& J, const DevScalars* sc, int dm, cudaStream_t st);
 template <typename T>
-cudaError_t launchg_copy_col(const T* src, T* dst, int64_t h, const DevScalars* sc, bool src_col, cudaStream_t st);
-template <typename T>
-cudaError_t launchg_scale(T* U, int64_t h, const DevScalars* sc, const double* scale, cudaStream_t st);
-cudaError_t launchg_loss(const double* c2, const DevScalars* sc, const double* nv2, double tau, int* flag,
-                         cudaStream_t st);
-cudaError_t launchg_inv_norm(const double* nv2, double* scale, DevScalars* sc, cudaStream_t st);
-cudaError_t launchg_qr_finish(const double* c1, const double* c2, const DevScalars* sc, int dm, const double* n0,
-                              const double* n1, double* Rm, double* out, double* scale, cudaStream_t st);
+cudaError_t launchg_scale(const GJobs<T>& J, const DevScalars* sc, cudaStream_t st);
+// flag = ||c2[:d]|| >= tau sqrt(c2[d]) (eq. loss_criterion; c2[d]: squared norm of the projected column)
+cudaError_t launchg_loss(const double* c2, const DevScalars* sc, double tau, int* flag, cudaStream_t st);
+// scale = 1 / norm from npart (nb entries); a zero or non-finite norm stops the solve
+cudaError_t launchg_inv_norm(const double* npart, int nb, double* scale, DevScalars* sc, cudaStream_t st);
 
 // Host-side preparation shared by the single and the batched handles (sgks_api.cu): the L
 // descriptor, the operator in the solver precision (CSR validation, value conversion, device
