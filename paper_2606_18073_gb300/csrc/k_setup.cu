@@ -151,9 +151,11 @@ __global__ void __launch_bounds__(kThreads) k_dots(const double* __restrict__ V0
     for (int c = threadIdx.x; c < k; c += kThreads) part[(size_t)blockIdx.x * k + c] = acc[c];
 }
 
-// the same for FP32 vectors, products in FP64
-__global__ void __launch_bounds__(kThreads) k_dots_f32(const float* __restrict__ V0, int64_t n, int k,
-                                                       const float* __restrict__ w, double* part) {
+// the same column after column, products in FP64: for FP32 vectors, and for a single column, where the
+// staged form would leave seven of its eight warps idle
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_dots_plain(const T* __restrict__ V0, int64_t n, int k,
+                                                         const T* __restrict__ w, double* part) {
     __shared__ double red[kWarps];
     for (int c = 0; c < k; ++c) {
         double a = 0.0;
@@ -162,7 +164,15 @@ __global__ void __launch_bounds__(kThreads) k_dots_f32(const float* __restrict__
         a = warp_sum(a);
         if (lane_id() == 0) red[warp_id()] = a;
         __syncthreads();
-        if (threadIdx.x == 0) part[(size_t)blockIdx.x * k + c] = tree_sumd<kWarps>(red);
+        if (threadIdx.x == 0) {   // the warps' sums with their rounding errors: all later columns carry this one's
+            double s = red[0], err = 0.0;
+            for (int q = 1; q < kWarps; ++q) {
+                const double t = s + red[q], bb = t - s;
+                err += (s - (t - bb)) + (red[q] - bb);
+                s = t;
+            }
+            part[(size_t)blockIdx.x * k + c] = s + err;
+        }
         __syncthreads();
     }
 }
@@ -196,13 +206,17 @@ __global__ void __launch_bounds__(kThreads) k_normalize(T* w, int64_t n, const d
         w[i] = (T)((double)w[i] * inv);
 }
 
-static void dots_go(const double* V0, int64_t n, int k, const double* w, double* part, int nb, cudaStream_t st) {
-    carveout_once((const void*)k_dots);
-    k_dots<<<nb, kThreads, sizeof(double) * (size_t)k, st>>>(V0, n, k, w, part);
-}
-static void dots_go(const float* V0, int64_t n, int k, const float* w, double* part, int nb, cudaStream_t st) {
-    carveout_once((const void*)k_dots_f32);
-    k_dots_f32<<<nb, kThreads, 0, st>>>(V0, n, k, w, part);
+template <typename T>
+static void dots_go(const T* V0, int64_t n, int k, const T* w, double* part, int nb, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8) {
+        if (k > 1) {
+            carveout_once((const void*)k_dots);
+            k_dots<<<nb, kThreads, sizeof(double) * (size_t)k, st>>>(V0, n, k, w, part);
+            return;
+        }
+    }
+    carveout_once((const void*)k_dots_plain<T>);
+    k_dots_plain<T><<<nb, kThreads, 0, st>>>(V0, n, k, w, part);
 }
 
 template <typename T>
