@@ -831,10 +831,11 @@ static cudaError_t csr_gradient_vv(const BDims& D, const DevA<T, V>& A, const De
 
 template <typename T, typename V>
 cudaError_t launchb_apply_column(const BDims& D, const DevA<T, V>& A, const DevL& L, const BBulk<T>& X,
-                                 const BSmall& S, cudaStream_t st) {
+                                 const BSmall& S, cudaStream_t st, bool a_rows) {
     if (A.kind == SGKS_OP_CSR) {
         constexpr int VW = vec_width<T>();
-        cudaError_t e = D.B >= VW ? csr_apply_vv<T, V, VW>(D, A, X, S, st)
+        cudaError_t e = !a_rows ? cudaSuccess
+                        : D.B >= VW ? csr_apply_vv<T, V, VW>(D, A, X, S, st)
                         : D.B == 2 ? csr_apply_vv<T, V, 2>(D, A, X, S, st)
                                    : csr_apply_vv<T, V, 1>(D, A, X, S, st);
         if (e != cudaSuccess) return e;
@@ -972,7 +973,7 @@ cudaError_t launchb_set_tol(DevScalars* sc, int B, double tol, cudaStream_t st) 
 
 #define SGKS_INST_B(T, V)                                                                                        \
     template cudaError_t launchb_apply_column<T, V>(const BDims&, const DevA<T, V>&, const DevL&, const BBulk<T>&, \
-                                                    const BSmall&, cudaStream_t);                                \
+                                                    const BSmall&, cudaStream_t, bool);                                \
     template cudaError_t launchb_gradient<T, V>(const BDims&, const DevA<T, V>&, const DevL&, const BBulk<T>&,     \
                                                 const BSmall&, T*, cudaStream_t);                                \
     template cudaError_t launchb_apply<T, V>(const BDims&, const DevA<T, V>&, const DevL&, int, const T*, T*,      \

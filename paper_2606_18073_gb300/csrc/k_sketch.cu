@@ -175,11 +175,8 @@ static cudaError_t launch_apply_column(const Dims& D, const DevA<T, V>& A, const
 
 template <typename T> struct GatherAcc { using type = T; };
 
-template <typename T, typename V>
-cudaError_t launch_sketch_column(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B,
-                                 const Small& S, const SketchCSR& SK, cudaStream_t st) {
-    cudaError_t e = launch_apply_column<T, V>(D, A, L, B, S, st);
-    if (e != cudaSuccess) return e;
+template <typename T>
+cudaError_t launch_sketch_gather_col(const Dims& D, const Bulk<T>& B, const Small& S, const SketchCSR& SK, cudaStream_t st) {
     carveout_once((const void*)k_sketch_gather_col<T, T, T>);
     return launch_pdl(k_sketch_gather_col<T, T, T>, 2 * D.s, kThreads, 0, st, D, (const T*)B.AW, (const T*)B.tmp_p, SK, S);
 }
@@ -202,15 +199,6 @@ cudaError_t launch_sketch_vec(const int32_t* ptr, const uint32_t* idx, const voi
         k_sketch_gather_vec<double, double><<<s, kThreads, 0, st>>>(ptr, idx, (const double*)v, out);
     }
     return cudaGetLastError();
-}
-
-template <typename T, typename V>
-cudaError_t launch_gaussian_sketch(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B,
-                                   const Small& S, const double* SA, const double* SL, const DenseWork& K,
-                                   cudaStream_t st) {
-    cudaError_t e = launch_apply_column<T, V>(D, A, L, B, S, st);
-    if (e != cudaSuccess) return e;
-    return launch_dense_pair<T, T>(D, B.AW, B.tmp_p, S, SA, SL, K, st);
 }
 
 // out[i] = scale * sum_{b < nb} part[b*len + i]: a warp per sum, lanes over the partials
@@ -329,7 +317,7 @@ cudaError_t build_sketch_csr(uint64_t key, int64_t h, int s, int zeta, int32_t* 
     return e;
 }
 
-// the apply half of launch_sketch_column alone (GKS appends A w and L w without a sketch)
+// A w -> column d of A W and L w -> tmp_p for the newest column w
 template <typename T, typename V>
 cudaError_t launch_apply_new_column(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B,
                                     const Small& S, cudaStream_t st) {
@@ -338,13 +326,11 @@ cudaError_t launch_apply_new_column(const Dims& D, const DevA<T, V>& A, const De
 
 #define SGKS_INST_SK(T, V)                                                                                  \
     template cudaError_t launch_apply_new_column<T, V>(const Dims&, const DevA<T, V>&, const DevL&,         \
-                                                       const Bulk<T>&, const Small&, cudaStream_t);         \
-    template cudaError_t launch_sketch_column<T, V>(const Dims&, const DevA<T, V>&, const DevL&,            \
-                                                    const Bulk<T>&, const Small&, const SketchCSR&,         \
-                                                    cudaStream_t);                                          \
-    template cudaError_t launch_gaussian_sketch<T, V>(const Dims&, const DevA<T, V>&, const DevL&,          \
-                                                      const Bulk<T>&, const Small&, const double*,          \
-                                                      const double*, const DenseWork&, cudaStream_t);
+                                                       const Bulk<T>&, const Small&, cudaStream_t);
+template cudaError_t launch_sketch_gather_col<float>(const Dims&, const Bulk<float>&, const Small&, const SketchCSR&,
+                                                     cudaStream_t);
+template cudaError_t launch_sketch_gather_col<double>(const Dims&, const Bulk<double>&, const Small&, const SketchCSR&,
+                                                      cudaStream_t);
 SGKS_INST_SK(float, float)
 SGKS_INST_SK(double, float)
 SGKS_INST_SK(double, double)

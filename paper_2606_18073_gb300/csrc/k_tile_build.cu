@@ -394,7 +394,7 @@ int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t 
                                         ray_seg);
     b.ran();
     if (b.e != cudaSuccess) return failed(b, why);
-    T = TiledA{TX, TY, nx, ny, nt, g.ntx, g.nty, g.ntiles, 4 * ngrp, order, tile_grp, goff, ray_ptr, ray_seg, ent};
+    T = TiledA{TX, TY, nx, ny, nt, g.ntx, g.nty, g.ntiles, 4 * ngrp, nseg, order, tile_grp, goff, ray_ptr, ray_seg, ent};
     return SGKS_OK;
 }
 
@@ -450,6 +450,42 @@ int build_tiles_t(const int32_t* trp, const int32_t* tci, const float* tval, int
     b.ran();
     if (b.e != cudaSuccess) return failed(b, why);
     T = TiledT{TX, TY, nx, ny, nt, g.ntx, g.nty, g.ntiles, order, tile_stage, tile_ray, ray, goff, stage, ent};
+    return SGKS_OK;
+}
+
+__global__ void k_tile_finite(const float* __restrict__ val, int64_t nnz, int* bad) {
+    bool b = false;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nnz; k += (int64_t)gridDim.x * blockDim.x)
+        b = b || !isfinite(val[k]);
+    if (b) *bad = 1;
+}
+
+int build_tiles64(const sgks_reg* reg, const int32_t* rp, const int32_t* ci, const float* val, const int32_t* trp,
+                  const int32_t* tci, const float* tval, int64_t m, int64_t n, int64_t nnz, int B, TiledA& T, TiledT& Tt,
+                  std::vector<void*>& allocs, cudaStream_t st, std::string* why) {
+    if (reg->kind == SGKS_REG_FD1 || nnz < (1 << 20)) return SGKS_OK;
+    const int nt = reg->kind == SGKS_REG_SPACETIME ? reg->nt : 1;
+    if ((int64_t)reg->nx * reg->ny * nt != n) return SGKS_OK;
+    {
+        Build b(st, &allocs);
+        int32_t* bad = b.temp<int32_t>(1);
+        b.zero(bad, 4);
+        if (b.e != cudaSuccess) return failed(b, why);
+        for (const float* v : {val, tval}) k_tile_finite<<<grid_for((nnz + 255) / 256), 256, 0, st>>>(v, nnz, bad);
+        b.ran();
+        const std::vector<int32_t> h = b.down(bad, 1);
+        if (b.e != cudaSuccess) return failed(b, why);
+        if (h[0]) return SGKS_OK;
+    }
+    TiledA a{};
+    TiledT t{};
+    int rc = build_tiles_t(trp, tci, tval, m, n, nnz, reg->nx, reg->ny, nt, tile_ty(B), tile_stage(B), t, allocs, st, why);
+    if (rc != SGKS_OK || !t.ntiles) return rc;
+    const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, B / kTileInst);
+    rc = build_tiles(rp, ci, val, m, n, nnz, reg->nx, reg->ny, nt, ctas < 4 * 152 ? 16 : 32, 16, a, allocs, st, why);
+    if (rc != SGKS_OK || !a.ntiles || a.nseg * 4 > nnz) return rc;
+    T = a;
+    Tt = t;
     return SGKS_OK;
 }
 

@@ -15,9 +15,11 @@
 #include <stdio.h>
 
 #include <atomic>
+#include <type_traits>
 #include <new>
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "sgks_internal.cuh"
@@ -119,6 +121,37 @@ struct Engine : EngineBase {
     const double* gSA = nullptr;
     const double* gSL = nullptr;
     DenseWork DW{};                 // of the dense sketches
+    // FP64 vectors on a ray operator: the tiled passes (k_tiles64.cu; ntiles = 0: the row kernels)
+    TiledA Ta{};
+    TiledT Tt{};
+    double* tpart = nullptr;        // [npart]
+
+    TileVec64 plain64(const T* v) const { return TileVec64{(const double*)v, 0, nullptr, 0, 1}; }
+    TileVec64 column64(const T* v, int64_t rows) const { return TileVec64{(const double*)v, rows, S.sc, D.dmax, 1}; }
+    // out = A v, A^T v or a stencil of v
+    cudaError_t op_apply(int which, const T* in, T* out) {
+        if constexpr (std::is_same<T, double>::value) {
+            if (Ta.ntiles && which == SGKS_APPLY_A)
+                return launch64_tile_apply(Ta, plain64(in), plain64(out), D.m, tpart, L, nullptr, st);
+            if (Ta.ntiles && which == SGKS_APPLY_AT)
+                return launch64_tile_gradient(Tt, plain64(in), plain64(out), nullptr, L, nullptr, nullptr, 0.0, st);
+        }
+        return launch_apply<T, V>(D, A, L, which, in, out, st);
+    }
+    // A w -> column d of A W, L w -> tmp_p for the newest column w
+    cudaError_t op_new_column() {
+        if constexpr (std::is_same<T, double>::value)
+            if (Ta.ntiles)
+                return launch64_tile_apply(Ta, column64(B.W, D.n), column64(B.AW, D.m), D.m, tpart, L, B.tmp_p, st);
+        return launch_apply_new_column<T, V>(D, A, L, B, S, st);
+    }
+    cudaError_t op_gradient_append() {
+        if constexpr (std::is_same<T, double>::value)
+            if (Ta.ntiles)
+                return launch64_tile_gradient(Tt, plain64(B.e), column64(B.W, D.n), S.sc, L, (const double*)B.x, nullptr,
+                                              D.lam, st);
+        return launch_gradient<T, V>(D, A, L, B, S, false, st);
+    }
     double* part_setup = nullptr;   // [nbS][8]
     int nbS = 1;
     int* d_err = nullptr;
@@ -168,13 +201,13 @@ struct Engine : EngineBase {
         }
         // W_0: orthonormal basis of K_l(A^T A, A^T b) (Sec. 2.1, Sec. 4), CGS2 on n-vectors
         T* W = B.W;
-        e = launch_apply<T, V>(D, A, L, SGKS_APPLY_AT, B.b, W, st);
+        e = op_apply(SGKS_APPLY_AT, B.b, W);
         if (e == cudaSuccess) e = launch_sqnorm<T>(W, D.n, part_setup, nbS, st);
         if (e == cudaSuccess) e = launch_normalize<T>(W, D.n, part_setup, nbS, st);
         for (int j = 1; j < D.ell && e == cudaSuccess; ++j) {
             T* wj = W + (size_t)j * D.n;
-            e = launch_apply<T, V>(D, A, L, SGKS_APPLY_A, W + (size_t)(j - 1) * D.n, B.tmp_m, st);
-            if (e == cudaSuccess) e = launch_apply<T, V>(D, A, L, SGKS_APPLY_AT, B.tmp_m, wj, st);
+            e = op_apply(SGKS_APPLY_A, W + (size_t)(j - 1) * D.n, B.tmp_m);
+            if (e == cudaSuccess) e = op_apply(SGKS_APPLY_AT, B.tmp_m, wj);
             for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
                 e = launch_dots<T>(W, D.n, j, wj, part_setup, nbS, st);
                 if (e == cudaSuccess) e = launch_orth_update<T>(wj, W, D.n, j, part_setup, nbS, st);
@@ -186,8 +219,10 @@ struct Engine : EngineBase {
     }
 
     cudaError_t sketch() {
-        if (gSA) return launch_gaussian_sketch<T, V>(D, A, L, B, S, gSA, gSL, DW, st);
-        return launch_sketch_column<T, V>(D, A, L, B, S, SK, st);
+        const cudaError_t e = op_new_column();
+        if (e != cudaSuccess) return e;
+        return gSA ? launch_dense_pair<T, T>(D, B.AW, B.tmp_p, S, gSA, gSL, DW, st)
+                   : launch_sketch_gather_col<T>(D, B, S, SK, st);
     }
 
     cudaError_t small_append(int d) {
@@ -212,7 +247,7 @@ struct Engine : EngineBase {
 
     cudaError_t launch_class(int cls) override {
         switch (cls) {
-            case PK_GRAD_APPEND: return launch_gradient<T, V>(D, A, L, B, S, false, st);
+            case PK_GRAD_APPEND: return op_gradient_append();
             case PK_SKETCH: return sketch();
             case PK_COMBINE_REFINE: return launch_combine<T>(D, B, S, 0, st);
             case PK_GRAD_REFINE: return launch_gradient<T, V>(D, A, L, B, S, true, st);
@@ -222,7 +257,7 @@ struct Engine : EngineBase {
 
     cudaError_t step() override {
         const int d = host_d;
-        cudaError_t e = timed(PK_GRAD_APPEND, d, [&] { return launch_gradient<T, V>(D, A, L, B, S, false, st); });
+        cudaError_t e = timed(PK_GRAD_APPEND, d, [&] { return op_gradient_append(); });
         if (e == cudaSuccess) e = timed(PK_SKETCH, d, [&] { return sketch(); });
         if (e == cudaSuccess) e = small_append(d);
         if (e == cudaSuccess) e = record_y(1, 0);
@@ -315,7 +350,7 @@ struct Engine : EngineBase {
 
     cudaError_t bw_apply(int which, const T* in, T* out) {
         g_launches.fetch_add(1);
-        return launch_apply<T, V>(D, A, L, which, in, out, st);
+        return op_apply(which, in, out);
     }
 
     cudaError_t bw_sketch_adj(bool isA, const double* u, T* out) {
@@ -545,7 +580,7 @@ struct Engine : EngineBase {
         if (which == SGKS_APPLY_SA || which == SGKS_APPLY_SL)
             return sketch_vector(which == SGKS_APPLY_SA, in, sizeof(T) == 4 ? SGKS_F32 : SGKS_F64, sizeof(T) == 4,
                                  (double*)out);
-        return launch_apply<T, V>(D, A, L, which, (const T*)in, (T*)out, st);
+        return launch_apply<T, V>(D, A, L, which, (const T*)in, (T*)out, st);   // full range: k_tiles64.cu
     }
 
     void* buffer(int which, size_t* elem_out, int64_t* rows, int64_t* ld) override {
@@ -632,7 +667,7 @@ struct EngineGKS : Engine<T, V> {
     cudaError_t append_gks(int d) {
         cudaError_t e = cudaSuccess;
         auto R = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-        R(timed(PK_SKETCH, d, [&] { return launch_apply_new_column<T, V>(D, A, L, B, S, st); }));
+        R(timed(PK_SKETCH, d, [&] { return Base::op_new_column(); }));
         R(timed(PK_QR_APPEND, d, [&] { return qr_cols(); }));
         R(timed(PK_STACKED_SOLVE, d, [&] { return launch_stacked_solve(D, S, st); }));
         return e;
@@ -650,7 +685,7 @@ struct EngineGKS : Engine<T, V> {
         const int d = host_d;
         // profile class 0 holds the gradient and its orthogonalisation against V
         cudaError_t e = timed(PK_GRAD_APPEND, d, [&] {
-            cudaError_t e2 = launch_gradient<T, V>(D, A, L, B, S, false, st);
+            cudaError_t e2 = Base::op_gradient_append();
             return e2 == cudaSuccess ? orth_new() : e2;
         });
         if (e == cudaSuccess) e = append_gks(d);
@@ -1200,6 +1235,16 @@ static int build_engine(sgks_handle* h, const sgks_op* op, const sgks_reg* reg, 
         std::string why;
         const int rc = prepare_operator<T, V>(op, E->A, h->allocs, E->d_err, h->st, &why);
         if (rc != SGKS_OK) return fail(h, rc, why);
+        if constexpr (std::is_same<T, double>::value && std::is_same<V, float>::value) {
+            if (op->kind == SGKS_OP_CSR) {
+                const int rt = build_tiles64(reg, E->A.rp, E->A.ci, E->A.val, E->A.trp, E->A.tci, E->A.tval, D.m, D.n, op->nnz, 1,
+                                             E->Ta, E->Tt, h->allocs, h->st, &why);
+                if (rt != SGKS_OK) return fail(h, rt, why);
+                if (E->Ta.ntiles) AL(E->tpart, E->Ta.npart);
+                if (e != cudaSuccess)
+                    return fail(h, SGKS_ERR_NOMEM, std::string("device allocation: ") + cudaGetErrorString(e));
+            }
+        }
         if (!gauss) {
             const int rs = prepare_sparse_sign(D.keyA, D.keyL, D.m, D.p, s, o.zeta, E->SK, h->allocs, E->d_err,
                                                h->st, &why);

@@ -112,10 +112,44 @@ struct Group : GroupBase {
     DevL L{};
     BBulk<T> X{};
     SketchCSR SK{};
+    // FP64 vectors on a ray operator: the tiled passes (k_tiles64.cu; ntiles = 0: the row kernels)
+    TiledA Ta{};
+    TiledT Tt{};
+    double* tpart = nullptr;    // [npart][B]
+
+    TileVec64 plain64(const T* v) const { return TileVec64{(const double*)v, 0, nullptr, 0, D.B}; }
+    TileVec64 column64(const T* v, int64_t rows) const {
+        return TileVec64{(const double*)v, rows * D.B, S.sc, D.dmax, D.B};
+    }
+    // out = A v or A^T v
+    cudaError_t op_apply(int which, const T* in, T* out) {
+        if constexpr (sizeof(T) == 8) {
+            if (Ta.ntiles && which == SGKS_APPLY_A)
+                return launch64_tile_apply(Ta, plain64(in), plain64(out), D.m, tpart, L, nullptr, st);
+            if (Ta.ntiles)
+                return launch64_tile_gradient(Tt, plain64(in), plain64(out), nullptr, L, nullptr, nullptr, 0.0, st);
+        }
+        return launchb_apply<T, V>(D, A, L, which, in, out, st);
+    }
+    cudaError_t op_new_column() {
+        if constexpr (sizeof(T) == 8)
+            if (Ta.ntiles) {
+                const cudaError_t e = launch64_tile_apply(Ta, column64(X.W, D.n), column64(X.AW, D.m), D.m, tpart, L, nullptr, st);
+                return e == cudaSuccess ? launchb_apply_column<T, V>(D, A, L, X, S, st, false) : e;
+            }
+        return launchb_apply_column<T, V>(D, A, L, X, S, st);
+    }
+    cudaError_t op_gradient(T* out) {
+        if constexpr (sizeof(T) == 8)
+            if (Ta.ntiles)
+                return launch64_tile_gradient(Tt, plain64(X.e), out ? plain64(out) : column64(X.W, D.n), S.sc, L,
+                                              (const double*)X.x, S.lam, 0.0, st);
+        return launchb_gradient<T, V>(D, A, L, X, S, out, st);
+    }
 
     cudaError_t sketch_column() {
         cudaError_t e = cudaSuccess;
-        RUNC(BK_APPLY, A.kind == SGKS_OP_CSR ? 2 : 1, (launchb_apply_column<T, V>(D, A, L, X, S, st)));
+        RUNC(BK_APPLY, A.kind == SGKS_OP_CSR ? (Ta.ntiles ? 3 : 2) : 1, op_new_column());
         RUNC(BK_GATHER, 1, launchb_sketch_gather<T>(D, X, SK, S, nullptr, nullptr, st));
         return e;
     }
@@ -130,7 +164,7 @@ struct Group : GroupBase {
     cudaError_t refine() {
         cudaError_t e = cudaSuccess;
         RUNC(BK_COMBINE_REFINE, 1, launchb_combine<T>(D, X, S, 0, st));
-        RUNC(BK_GRAD_REFINE, 1, (launchb_gradient<T, V>(D, A, L, X, S, X.r, st)));
+        RUNC(BK_GRAD_REFINE, 1, op_gradient(X.r));
         RUNC(BK_GRAD_REFINE, 1, launchb_wtr<T>(D, X, S, X.r, st));
         RUNC(BK_REFINE_SOLVE, 1, launch_refine_solve2(Ds, Small{}, st, Sarr, D.B, D.nb_refine));
         return e;
@@ -158,12 +192,12 @@ struct Group : GroupBase {
         }
         T* W = X.W;
         const size_t col = (size_t)D.n * B;
-        RUN(1, (launchb_apply<T, V>(D, A, L, SGKS_APPLY_AT, X.b, W, st)));
+        RUN(1, op_apply(SGKS_APPLY_AT, X.b, W));
         if (e == cudaSuccess) e = normalize(W);
         for (int j = 1; j < D.ell && e == cudaSuccess; ++j) {
             T* wj = W + j * col;
-            RUN(1, (launchb_apply<T, V>(D, A, L, SGKS_APPLY_A, W + (j - 1) * col, X.tm, st)));
-            RUN(1, (launchb_apply<T, V>(D, A, L, SGKS_APPLY_AT, X.tm, wj, st)));
+            RUN(Ta.ntiles ? 2 : 1, op_apply(SGKS_APPLY_A, W + (j - 1) * col, X.tm));
+            RUN(1, op_apply(SGKS_APPLY_AT, X.tm, wj));
             for (int pass = 0; pass < 2; ++pass) {
                 RUN(2, launchb_dots<T>(D, W, j, wj, S, st));
                 RUN(1, launchb_vec_update<T>(D, wj, W, j, S, 0, st));
@@ -182,7 +216,7 @@ struct Group : GroupBase {
     // one iteration of Algorithm 2 for every live instance of the group
     cudaError_t step() override {
         cudaError_t e = cudaSuccess;
-        RUNC(BK_GRAD_APPEND, 1, (launchb_gradient<T, V>(D, A, L, X, S, nullptr, st)));
+        RUNC(BK_GRAD_APPEND, 1, op_gradient(nullptr));
         if (e == cudaSuccess) e = sketch_column();
         if (e == cudaSuccess) e = small_append();
         for (int r = 0; r < n_refine && e == cudaSuccess; ++r) e = refine();
@@ -242,7 +276,7 @@ struct Group : GroupBase {
             D.slice_kb = tune_pick(best, pick, t_def, def);
             D.nb_combine = batch_combine_grid(D, sizeof(T));
         }
-        if (A.kind == SGKS_OP_CSR) {
+        if (A.kind == SGKS_OP_CSR && !Ta.ntiles) {   // tiled passes have no lanes to tune
             for (int which = 0; which < 2; ++which) {
                 int* field = which == 0 ? &D.nl_a : &D.nl_t;
                 float best = 1e30f, t_def = 0.f;
@@ -778,8 +812,17 @@ int build_groups(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const st
     const int dmax = o.ell + o.max_iters;
     if (o.n_refine > 0 && batch_refine_smem(dmax, 1, sizeof(T)) > 200 * 1024)
         return bfail(h, SGKS_ERR_INVALID, "ell + max_iters too large for the batched refinement");
+    const std::vector<int> sizes = split_groups(inst.size(), max_group_size(dmax, o.n_refine, sizeof(T)));
+    TiledA Ta{};
+    TiledT Tt{};
+    if constexpr (sizeof(T) == 8 && sizeof(V) == 4)
+        if (op->kind == SGKS_OP_CSR && !(o.flags & SGKS_FLAG_NO_TILES)) {
+            rc = build_tiles64(reg, A.rp, A.ci, A.val, A.trp, A.tci, A.tval, op->m, op->n, op->nnz, sizes[0], Ta, Tt, h->allocs,
+                               h->st, &why);
+            if (rc != SGKS_OK) return bfail(h, rc, why);
+        }
     size_t pos = 0;
-    for (const int B : split_groups(inst.size(), max_group_size(dmax, o.n_refine, sizeof(T)))) {
+    for (const int B : sizes) {
         Group<T, V>* G = new (std::nothrow) Group<T, V>();
         if (!G) return bfail(h, SGKS_ERR_NOMEM, "host allocation failed");
         h->groups.push_back(G);
@@ -814,6 +857,9 @@ int build_groups(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const st
         BA(X.tp, pB);
         BA(X.tm, mB);
         if (o.n_refine > 0) BA(X.r, nB);
+        G->Ta = Ta;
+        G->Tt = Tt;
+        if (Ta.ntiles) BA(G->tpart, (size_t)Ta.npart * B);
 #undef BA
         if (e != cudaSuccess) return bfail(h, SGKS_ERR_NOMEM, std::string("device allocation: ") + cudaGetErrorString(e));
         e = cudaMemsetAsync(X.xs, 0, sizeof(T) * nB, h->st);

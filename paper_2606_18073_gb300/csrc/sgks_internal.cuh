@@ -816,13 +816,9 @@ struct Dims {
     int max_iters;
 };
 
-template <typename T, typename V>
-cudaError_t launch_sketch_column(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B,
-                                 const Small& S, const SketchCSR& SK, cudaStream_t st);
-template <typename T, typename V>
-cudaError_t launch_gaussian_sketch(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B,
-                                   const Small& S, const double* SA, const double* SL, const DenseWork& K,
-                                   cudaStream_t st);
+// S_A (A W[:, d]) and S_L t from the column d of A W and the scratch t = L w
+template <typename T>
+cudaError_t launch_sketch_gather_col(const Dims& D, const Bulk<T>& B, const Small& S, const SketchCSR& SK, cudaStream_t st);
 // part and cnt elements of the DenseWork of an s x m and an s x p sketch
 void dense_work_size(int64_t m, int64_t p, int s, size_t* part, size_t* cnt);
 template <typename TA, typename TL>
@@ -966,7 +962,7 @@ struct PtrPack {
 
 template <typename T, typename V>
 cudaError_t launchb_apply_column(const BDims& D, const DevA<T, V>& A, const DevL& L, const BBulk<T>& X,
-                                 const BSmall& S, cudaStream_t st);
+                                 const BSmall& S, cudaStream_t st, bool a_rows = true);
 template <typename T>
 cudaError_t launchb_sketch_gather(const BDims& D, const BBulk<T>& X, const SketchCSR& SK, const BSmall& S,
                                   const T* vec, double* out_vec, cudaStream_t st);
@@ -999,6 +995,7 @@ cudaError_t launchb_scatter_out(const T* in, const PtrPack& P, int64_t len, int 
 struct TiledA {
     int TX, TY, nx, ny, nt, ntx, nty, ntiles;
     int64_t npart;             // segment positions: rows of the partial sums
+    int64_t nseg;              // segments, without the filling
     const int32_t* order;      // tiles by descending work, so that the last CTAs are the short ones
     const int32_t* tile_grp;   // [ntiles + 1]
     const int32_t* goff;       // [npart / 4 + 1]
@@ -1036,6 +1033,31 @@ int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t 
                 int nt, int TX, int TY, TiledA& T, std::vector<void*>& allocs, cudaStream_t st, std::string* why);
 int build_tiles_t(const int32_t* trp, const int32_t* tci, const float* tval, int64_t m, int64_t n, int64_t nnz, int nx,
                   int ny, int nt, int TY, int stage, TiledT& T, std::vector<void*>& allocs, cudaStream_t st, std::string* why);
+// Vectors of B interleaved instances for the FP64 tiled passes (k_tiles64.cu): p[q B + b], or, with
+// scalars, column sc[b].d of p (columns of `col` values).
+struct TileVec64 {
+    const double* p;
+    int64_t col;
+    const DevScalars* sc;   // null: a plain vector
+    int dmax, B;
+    // instance b's vector (element q at [q B]); null when the instance has stopped or its basis is full
+    __device__ __forceinline__ const double* column(int b) const {
+        if (!sc) return p + b;
+        return !sc[b].stop && sc[b].d < dmax ? p + (size_t)sc[b].d * col + b : nullptr;
+    }
+};
+// U = A W through the tiles (part: npart x B doubles); lw (single handle): L w too, else null
+cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, double* part,
+                                const DevL& L, double* lw, cudaStream_t st);
+// O = A^T E + lambda L^T L x (x null: A^T E); lambda per instance (lam) or one (lam1).  O without scalars but
+// sc given: instances that have stopped are left out.
+cudaError_t launch64_tile_gradient(const TiledT& T, const TileVec64& E, const TileVec64& O, DevScalars* sc, const DevL& L,
+                                   const double* x, const double* lam, double lam1, cudaStream_t st);
+// Both layouts for FP64 vectors where they pay: a CSR operator with finite FP32 values and 2^20 entries or more
+// on an image (the regularizer's), whose rows share tiles; else T.ntiles = Tt.ntiles = 0.  B: largest group.
+int build_tiles64(const sgks_reg* reg, const int32_t* rp, const int32_t* ci, const float* val, const int32_t* trp,
+                  const int32_t* tci, const float* tval, int64_t m, int64_t n, int64_t nnz, int B, TiledA& T, TiledT& Tt,
+                  std::vector<void*>& allocs, cudaStream_t st, std::string* why);
 int tile_instances(const BDims& D);   // instances per CTA of the forward pass
 // u_i = A w_i into column d_i of AW through the tiles (partials in part, npart x B float-float)
 template <typename TW>
