@@ -7,7 +7,7 @@
 // CTA keeps the gathered side in shared memory:
 //   forward    a tile of w (IC instances); the CTA walks the (ray, tile) segments that cross the tile
 //              and leaves one float-float partial per segment and instance, which kbx_seg_reduce adds
-//              up ray by ray in the order of the row's entries;
+//              up ray by ray;
 //   transposed the rays that cross a tile are staged in shared memory a few hundred at a time (rays of a
 //              tile in ascending order) and every pixel of the tile adds its entries of the stage to
 //              accumulators that stay in registers; the stencil and lambda finish the row, so the
@@ -182,13 +182,14 @@ __global__ void __launch_bounds__(Lanes<IC>::threads, IC >= 16 ? 3 : 2) kbx_tile
     }
 }
 
-// u_i = sum over the ray's segments, in the order of the row's entries, of the partials -> column
-// d_i of AW.  NB = 2: a thread takes two instances, partials as (hi0, hi1, lo0, lo1).
+// u_i = sum over the ray's segments of the partials -> column d_i of AW.  NB = 2: a thread takes two
+// instances, partials as (hi0, hi1, lo0, lo1).  `lanes` neighbouring lanes share a ray (seg_lanes), each
+// with its own accumulator, merged in a fixed tree.
 template <typename TW, int NB>
 __global__ void __launch_bounds__(kThreads) kbx_seg_reduce(BDims D, TiledA T, BBulkX<TW> X, BSmall S,
-                                                           const float2* __restrict__ part) {
-    const int B = D.B, H = B / NB;
-    const int b = (threadIdx.x & (H - 1)) * NB;
+                                                           const float2* __restrict__ part, int lanes) {
+    const int B = D.B, H = B / NB, G = H * lanes;
+    const int b = (threadIdx.x & (H - 1)) * NB, s = (threadIdx.x & (G - 1)) / H;
     float2* out[NB];
     bool any = false;
 #pragma unroll
@@ -197,29 +198,36 @@ __global__ void __launch_bounds__(kThreads) kbx_seg_reduce(BDims D, TiledA T, BB
         out[v] = (!sc.stop && sc.d < D.dmax) ? X.AW + (size_t)sc.d * D.m * B + b + v : nullptr;
         any = any || out[v];
     }
-    if (!any) return;
-    for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t < D.m * H; t += gstride()) {
-        const int64_t r = qdiv(t, H);
-        const int k0 = T.ray_ptr[r], k1 = T.ray_ptr[r + 1];
+    if (!__any_sync(0xffffffffu, any)) return;
+    const int64_t tot = D.m * G;
+    for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t - lane_id() < tot; t += gstride()) {
+        const int64_t r = qdiv(t, G);
+        const bool in = t < tot && any;
+        const int k0 = in ? T.ray_ptr[r] + s : 0, k1 = in ? T.ray_ptr[r + 1] : 0;
+        int c = 0;
+        Dot2 a[NB];
         if constexpr (NB == 2) {
-            Dot2x2 a;
-#pragma unroll 4
-            for (int k = k0; k < k1; ++k) {
+            Dot2x2 q;
+#pragma unroll 8
+            for (int k = k0; k < k1; k += lanes) {
                 const float4 f = __ldcs(reinterpret_cast<const float4*>(part + (size_t)T.ray_seg[k] * B + b));
-                a.accumulate(pack2(f.x, f.y), pack2(f.z, f.w));
-                if ((k - k0) % 4 == 3) a.renorm();   // ff.cuh: free, the loads set the pace
+                q.accumulate(pack2(f.x, f.y), pack2(f.z, f.w));
+                if (++c % 4 == 0) q.renorm();   // ff.cuh: free, the loads set the pace
             }
-            if (out[0]) out[0][r * B] = a.half(0).value();
-            if (out[NB - 1]) out[NB - 1][r * B] = a.half(1).value();
+            a[0] = q.half(0);
+            a[1] = q.half(1);
         } else {
-            Dot2 a;
-#pragma unroll 4
-            for (int k = k0; k < k1; ++k) {
+#pragma unroll 8
+            for (int k = k0; k < k1; k += lanes) {
                 const float2 v = __ldcs(part + (size_t)T.ray_seg[k] * B + b);
-                a.add2(v.x, v.y);
-                if ((k - k0) % 4 == 3) a.renorm();
+                a[0].add2(v.x, v.y);
+                if (++c % 4 == 0) a[0].renorm();
             }
-            if (out[0]) out[0][r * B] = a.value();
+        }
+#pragma unroll
+        for (int v = 0; v < NB; ++v) {
+            for (int off = H; off < G; off <<= 1) dot2_xor_merge(a[v], off);
+            if (out[v] && in && s == 0) out[v][r * B] = a[v].value();
         }
     }
 }
@@ -360,8 +368,9 @@ static cudaError_t tile_apply_ic(const BDims& D, const TiledA& T, const BBulkX<T
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     constexpr int NB = IC == 1 ? 1 : 2;
-    const int64_t rb = (D.m * (D.B / NB) + kThreads - 1) / kThreads;
-    kbx_seg_reduce<TW, NB><<<(int)std::max<int64_t>(1, std::min<int64_t>(rb, 8 * 152)), kThreads, 0, st>>>(D, T, X, S, part);
+    const int lanes = seg_lanes(D.B / NB, D.alone);
+    const int64_t rb = (D.m * (D.B / NB) * lanes + kThreads - 1) / kThreads;
+    kbx_seg_reduce<TW, NB><<<(int)std::max<int64_t>(1, std::min<int64_t>(rb, 8 * 152)), kThreads, 0, st>>>(D, T, X, S, part, lanes);
     return cudaGetLastError();
 }
 

@@ -108,10 +108,11 @@ __global__ void __launch_bounds__(kThreads, 4) kd_tile_apply(TiledA T, TileVec64
     }
 }
 
-// u_i = 2^448 sum over the ray's segments, in the order of the row's entries; then, where lw is given
-// (single handle), t = L w, a row per thread
+// u_i = 2^448 sum over the ray's segments; then, where lw is given (single handle), t = L w, a row per
+// thread.  Latency: a lane waits for the segment's number, then for its partial, so `lanes` (seg_lanes)
+// neighbouring ones share a ray.
 __global__ void __launch_bounds__(kThreads) kd_seg_reduce(TiledA T, TileVec64 U, int64_t m, const double* __restrict__ part,
-                                                          int nbu, DevL L, TileVec64 W, double* lw) {
+                                                          int lanes, int nbu, DevL L, TileVec64 W, double* lw) {
     pdl_wait();
     if ((int)blockIdx.x >= nbu) {
         const double* w = W.column(0);
@@ -121,15 +122,20 @@ __global__ void __launch_bounds__(kThreads) kd_seg_reduce(TiledA T, TileVec64 U,
             lw[j] = l_row<double>(L, j, w);
         return;
     }
-    const int B = U.B, b = threadIdx.x & (B - 1);
+    const int B = U.B, b = threadIdx.x & (B - 1), G = B * lanes;
     double* u = const_cast<double*>(U.column(b));
-    if (!u) return;
-    for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t < m * B; t += (int64_t)nbu * kThreads) {
-        const int64_t r = qdiv(t, B);
+    if (!__any_sync(0xffffffffu, u != nullptr)) return;
+    const int s = (threadIdx.x & (G - 1)) / B;
+    const int64_t tot = m * G;
+    for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t - lane_id() < tot; t += (int64_t)nbu * kThreads) {
+        const int64_t r = qdiv(t, G);
+        const bool in = t < tot && u;
         double a = 0.0;
+        const int k1 = in ? T.ray_ptr[r + 1] : 0;
 #pragma unroll 4
-        for (int k = T.ray_ptr[r]; k < T.ray_ptr[r + 1]; ++k) a += __ldcs(part + (size_t)T.ray_seg[k] * B + b);
-        u[r * B] = a * kHalfScale;
+        for (int k = in ? T.ray_ptr[r] + s : 0; k < k1; k += lanes) a += __ldcs(part + (size_t)T.ray_seg[k] * B + b);
+        for (int off = B; off < G; off <<= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        if (in && s == 0) u[r * B] = a * kHalfScale;
     }
 }
 
@@ -217,7 +223,7 @@ static cudaError_t apply64_ic(const TiledA& T, const TileVec64& W, double* part,
     return launch_pdl(k, (unsigned)(ctas * split), kThreads, smem, st, T, W, split, part);
 }
 
-cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, double* part,
+cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, int lanes, double* part,
                                 const DevL& L, double* lw, cudaStream_t st) {
     cudaError_t e;
     switch (std::min(W.B, kTileInst)) {
@@ -228,9 +234,9 @@ cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileV
         default: e = apply64_ic<16>(T, W, part, st); break;
     }
     if (e != cudaSuccess) return e;
-    const int nbu = (int)std::max<int64_t>(1, std::min<int64_t>((m * W.B + kThreads - 1) / kThreads, 8 * 152));
+    const int nbu = (int)std::max<int64_t>(1, std::min<int64_t>((m * W.B * lanes + kThreads - 1) / kThreads, 8 * 152));
     const int nbl = lw ? (int)std::max<int64_t>(1, std::min<int64_t>((L.p + kThreads - 1) / kThreads, 8 * 152)) : 0;
-    return launch_pdl(kd_seg_reduce, nbu + nbl, kThreads, 0, st, T, U, m, part, nbu, L, W, lw);
+    return launch_pdl(kd_seg_reduce, nbu + nbl, kThreads, 0, st, T, U, m, part, lanes, nbu, L, W, lw);
 }
 
 template <int IC, int TY>

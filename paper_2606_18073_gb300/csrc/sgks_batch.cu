@@ -125,7 +125,7 @@ struct Group : GroupBase {
     cudaError_t op_apply(int which, const T* in, T* out) {
         if constexpr (sizeof(T) == 8) {
             if (Ta.ntiles && which == SGKS_APPLY_A)
-                return launch64_tile_apply(Ta, plain64(in), plain64(out), D.m, tpart, L, nullptr, st);
+                return launch64_tile_apply(Ta, plain64(in), plain64(out), D.m, seg_lanes(D.B, D.alone), tpart, L, nullptr, st);
             if (Ta.ntiles)
                 return launch64_tile_gradient(Tt, plain64(in), plain64(out), nullptr, L, nullptr, nullptr, 0.0, st);
         }
@@ -134,7 +134,7 @@ struct Group : GroupBase {
     cudaError_t op_new_column() {
         if constexpr (sizeof(T) == 8)
             if (Ta.ntiles) {
-                const cudaError_t e = launch64_tile_apply(Ta, column64(X.W, D.n), column64(X.AW, D.m), D.m, tpart, L, nullptr, st);
+                const cudaError_t e = launch64_tile_apply(Ta, column64(X.W, D.n), column64(X.AW, D.m), D.m, seg_lanes(D.B, D.alone), tpart, L, nullptr, st);
                 return e == cudaSuccess ? launchb_apply_column<T, V>(D, A, L, X, S, st, false) : e;
             }
         return launchb_apply_column<T, V>(D, A, L, X, S, st);
@@ -668,6 +668,7 @@ int init_group(sgks_batch* h, GroupBase* G, const sgks_op* op, const DevL& L, in
     D.nl_a = 8;
     D.nl_t = 8;
     D.tile_ic = 0;
+    D.alone = true;   // set once all groups are there
     D.nb_combine = comb_grid(D);
     // SGKS_TEST_TIMEOUT_GROUP=g (read at create) gives group g's bulk-copy combine a wait limit of
     // zero rounds: its first wait reports a timeout, the CTA drains its own copies with the full
@@ -1116,6 +1117,7 @@ int sgks_batch_create(sgks_batch** hp, int32_t count, const sgks_op* A, const sg
             rc = build_groups<double, float>(h, op, reg, members[k], b, lambdas, x_true, sketch_rows, seed, o,
                                              cluster2);
     }
+    for (GroupBase* g : h->groups) g->D.alone = h->groups.size() == 1;
     if (rc == SGKS_OK && h->groups.size() > 1) {
         for (size_t g = 0; g < h->groups.size() && e == cudaSuccess; ++g) {
             cudaStream_t s = nullptr;

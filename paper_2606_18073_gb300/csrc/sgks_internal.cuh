@@ -910,6 +910,7 @@ struct BDims {
     int nl_a, nl_t;           // CSR rows: lanes per row of A and of A^T (powers of two <= 32, tuned)
     int nb_refine;            // CTAs of kb_wtr (each leaves one partial per instance)
     int nb_setup;             // CTAs of the setup reductions
+    bool alone;               // the batch's only group
     int tile_ic;              // tiled forward pass: instances per CTA (0: kTileInst; tuned)
     int wait_tries;           // bounded waits of the bulk-copy combine's ring (kWaitTries; 0 in the
                               // timeout test of SGKS_TEST_TIMEOUT_GROUP, see sgks_batch.cu)
@@ -959,6 +960,13 @@ struct BSmall {
 struct PtrPack {
     const void* p[kMaxBatch];
 };
+
+// Lanes that share a ray of n instance lanes in the sums over segments, within a warp: a ray of a CT image crosses
+// some 20 to 60 tiles, and eight lanes leave each one round or two of loads.  512^2, FP64, one vector: 45 -> 20 us;
+// a batch of one, float-float, 301^2: 17 -> 11 us.  A batch of several groups runs them next to each other and
+// fills the chip without, where merging costs more than waiting (7.61 against 7.72 ms per solve of 11 slices of
+// 243^2): one lane there.
+inline int seg_lanes(int n, bool alone) { return !alone || n >= 32 ? 1 : std::min(8, 32 / n); }
 
 template <typename T, typename V>
 cudaError_t launchb_apply_column(const BDims& D, const DevA<T, V>& A, const DevL& L, const BBulk<T>& X,
@@ -1047,7 +1055,7 @@ struct TileVec64 {
     }
 };
 // U = A W through the tiles (part: npart x B doubles); lw (single handle): L w too, else null
-cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, double* part,
+cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, int lanes, double* part,
                                 const DevL& L, double* lw, cudaStream_t st);
 // O = A^T E + lambda L^T L x (x null: A^T E); lambda per instance (lam) or one (lam1).  O without scalars but
 // sc given: instances that have stopped are left out.
