@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kThreads) k_combine(Dims D, Bulk<T> B, Small S
     __shared__ int am_last;
     DevScalars* sc = S.sc;
     if (sc->stop) return;
-    const int d = sc->d;
+    const int d = sc->d, iter = sc->iter;
     for (int j = threadIdx.x; j < D.dmax + kCombCols; j += kThreads) ys[j] = j < d ? (T)S.y[j] : T(0);
     const int tid = threadIdx.x;
     const bool isx = (int)blockIdx.x < nbx;
@@ -304,44 +304,42 @@ __global__ void __launch_bounds__(kThreads) k_combine(Dims D, Bulk<T> B, Small S
             for (int v = 0; v < VW; ++v) B.e[i0 + v] = acc[v] - B.b[i0 + v];
         }
     }
-    if (mode == 0) return;
-    // block partials of the three squared norms: warp sums in the solver precision, the
-    // 8 warp values combined in FP64 by three threads
-    const T w0 = warp_sum(q0), w1 = warp_sum(q1), w2 = warp_sum(q2);
-    if (lane_id() == 0) { red[0][warp_id()] = (double)w0; red[1][warp_id()] = (double)w1; red[2][warp_id()] = (double)w2; }
+    if (mode == 0 || !isx) return;
+    // block partials of the three squared norms, of the CTAs that hold x: warp sums in the solver precision
+    // (three at once: six steps instead of fifteen), the 8 warp values combined in FP64 by three threads
+    const int lane = lane_id(), warp = warp_id();
+    T q[4] = {q0, q1, q2, T(0)};
+    const T wq = warp_sum_rows<4>(q);   // lanes 8 k .. 8 k + 7: the sum of q[k]
+    if (lane < 24 && (lane & 7) == 0) red[lane >> 3][warp] = (double)wq;
     __syncthreads();
-    if (tid < 3) S.kapart[(size_t)blockIdx.x * 3 + tid] = tree_sumd<kWarps>(red[tid]);
-    __threadfence();
+    if (tid < 3) {
+        S.kapart[(size_t)blockIdx.x * 3 + tid] = tree_sumd<kWarps>(red[tid]);
+        __threadfence();
+    }
     __syncthreads();
-    if (tid == 0) am_last = (atomicAdd(&sc->ka_done, 1) == (int)gridDim.x - 1);
+    if (tid == 0) am_last = (atomicAdd(&sc->ka_done, 1) == nbx - 1);
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    // last CTA: fixed-order reduction of the partials (warp q sums quantity q)
-    if (warp_id() < 3) {   // warp q reduces quantity q over the CTA partials (fixed order)
-        const int q = warp_id();
-        double t = 0.0;
-        for (int b = lane_id(); b < (int)gridDim.x; b += 32) t += __ldcg(S.kapart + (size_t)b * 3 + q);
-        t = warp_sum(t);
-        if (lane_id() == 0) red[q][0] = t;
+    // last CTA: warp q sums quantity q over the CTA partials (fixed order); the two quotients in two warps
+    if (warp < 3) {
+        const double t = warp_sum_parts(S.kapart + warp, nbx, 3);
+        if (lane == 0) red[warp][0] = t;
     }
     __syncthreads();
+    const double dx2 = red[0][0], xo2 = red[1][0];
+    if (tid == 32) {   // RRE, with the values that thread 0 does not write
+        const double rre = B.xtrue ? sqrt(red[2][0] / sc->xt2) : (double)NAN;
+        if (mode == 2) sc->rre0 = rre;
+        else if (iter < D.max_iters) S.rre_hist[iter] = rre;
+        sc->rre_last = rre;
+    }
     if (tid == 0) {
-        const double dx2 = red[0][0], xo2 = red[1][0], er2 = red[2][0];
-        const double rre = B.xtrue ? sqrt(er2 / sc->xt2) : (double)NAN;
-        if (mode == 2) {
-            sc->rre0 = rre;
-            sc->rre_last = rre;
-        } else {
+        if (mode != 2) {
             const double rc = sqrt(dx2 / xo2);
-            const int k = sc->iter;
-            if (k < D.max_iters) {
-                S.rc_hist[k] = rc;
-                S.rre_hist[k] = rre;
-            }
+            if (iter < D.max_iters) S.rc_hist[iter] = rc;
             sc->rc_last = rc;
-            sc->rre_last = rre;
-            sc->iter = k + 1;
+            sc->iter = iter + 1;
             if (sc->tol_on && rc < sc->tol) {
                 sc->status = ST_STOPPED;
                 sc->stop = 1;

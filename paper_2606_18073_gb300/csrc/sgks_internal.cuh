@@ -205,8 +205,8 @@ __device__ __forceinline__ double warp_sum_acc(T v) { return (double)warp_sum(v)
 
 // Sums over the warp of R values per lane: at each step half of the lanes take over half of the
 // values, until a lane holds one row's sum; lane & (32 / R - 1) == 0 then holds row lane / (32 / R).
-template <int R>
-__device__ __forceinline__ double warp_sum_rows(double (&a)[R]) {
+template <int R, typename T>
+__device__ __forceinline__ T warp_sum_rows(T (&a)[R]) {
     const int lane = lane_id();
     int off = 16;
 #pragma unroll
@@ -214,11 +214,11 @@ __device__ __forceinline__ double warp_sum_rows(double (&a)[R]) {
         const bool up = (lane & off) != 0;
 #pragma unroll
         for (int i = 0; i < h; ++i) {
-            const double keep = up ? a[i + h] : a[i], send = up ? a[i] : a[i + h];
+            const T keep = up ? a[i + h] : a[i], send = up ? a[i] : a[i + h];
             a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
         }
     }
-    double v = a[0];
+    T v = a[0];
     for (; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     return v;
 }
