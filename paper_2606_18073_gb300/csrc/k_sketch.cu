@@ -80,20 +80,20 @@ __device__ __forceinline__ double as_double(T v) { return (double)v; }
 template <>
 __device__ __forceinline__ double as_double<float2>(float2 v) { return (double)v.x + (double)v.y; }
 
-// Sum of sign_k v[col_k] over the entries [b, e) of one sketch row; CTA-wide, fixed order.
+// the next eight entries of the thread, from entry k0 on
+__device__ __forceinline__ void load_entries(const uint32_t* __restrict__ idx, int k0, int e, uint32_t (&u)[8]) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) u[q] = k0 + q * kThreads < e ? __ldg(idx + k0 + q * kThreads) : 0u;
+}
+
+// Sum of sign_k v[col_k] over the entries [b, e) of one sketch row, u: the thread's first ones; CTA-wide, fixed order.
 template <typename Acc, typename TV>
 __device__ __forceinline__ double gather_row(const uint32_t* __restrict__ idx, int b, int e, const TV* __restrict__ v,
-                                             double* red) {
+                                             double* red, uint32_t (&u)[8]) {
     // eight entries per thread per round: their indices first, then the eight gathers, then the
     // sum in entry order (an S_L row of the 256^2 problem has ~2,600 entries, ten per thread)
     Acc a = Acc(0);
     for (int k0 = b + (int)threadIdx.x; k0 < e; k0 += 8 * kThreads) {
-        uint32_t u[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int k = k0 + q * kThreads;
-            u[q] = k < e ? __ldg(idx + k) : 0u;
-        }
         Acc val[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q)
@@ -101,6 +101,7 @@ __device__ __forceinline__ double gather_row(const uint32_t* __restrict__ idx, i
 #pragma unroll
         for (int q = 0; q < 8; ++q)
             if (k0 + q * kThreads < e) a += (u[q] >> 31) ? -val[q] : val[q];
+        load_entries(idx, k0 + 8 * kThreads, e, u);
     }
     const double t = warp_sum_acc(a);
     if (lane_id() == 0) red[warp_id()] = t;
@@ -113,18 +114,20 @@ __device__ __forceinline__ double gather_row(const uint32_t* __restrict__ idx, i
 template <typename TA, typename TL, typename Acc>
 __global__ void __launch_bounds__(kThreads) k_sketch_gather_col(Dims D, const TA* __restrict__ AW, const TL* __restrict__ lw,
                                                                 SketchCSR SK, Small S) {
+    __shared__ double red[kWarps];
+    const bool isA = (int)blockIdx.x < D.s;
+    const int r = isA ? blockIdx.x : blockIdx.x - D.s;
+    const uint32_t* idx = isA ? SK.idxA : SK.idxL;   // fixed since the handle's creation: read before the wait
+    const int b = (isA ? SK.ptrA : SK.ptrL)[r], e = (isA ? SK.ptrA : SK.ptrL)[r + 1];
+    uint32_t u[8];
+    load_entries(idx, b + (int)threadIdx.x, e, u);
     pdl_wait();   // all global reads below depend on the previous kernel
     pdl_trigger();   // the QR append loads its earlier columns meanwhile
-    __shared__ double red[kWarps];
     const DevScalars* sc = S.sc;
     if (sc->stop) return;
     const int d = sc->d;
     if (d >= D.dmax) return;
-    const bool isA = (int)blockIdx.x < D.s;
-    const int r = isA ? blockIdx.x : blockIdx.x - D.s;
-    double v;
-    if (isA) v = gather_row<Acc>(SK.idxA, SK.ptrA[r], SK.ptrA[r + 1], AW + (size_t)d * D.m, red);
-    else v = gather_row<Acc>(SK.idxL, SK.ptrL[r], SK.ptrL[r + 1], lw, red);
+    const double v = isA ? gather_row<Acc>(idx, b, e, AW + (size_t)d * D.m, red, u) : gather_row<Acc>(idx, b, e, lw, red, u);
     if (threadIdx.x == 0) (isA ? S.partA : S.partL)[r] = v;
 }
 
@@ -135,7 +138,9 @@ __global__ void __launch_bounds__(kThreads) k_sketch_gather_vec(const int32_t* _
                                                                 const TV* __restrict__ v, double* out) {
     __shared__ double red[kWarps];
     const int r = blockIdx.x;
-    const double t = gather_row<Acc>(idx, ptr[r], ptr[r + 1], v, red);
+    uint32_t u[8];
+    load_entries(idx, ptr[r] + (int)threadIdx.x, ptr[r + 1], u);
+    const double t = gather_row<Acc>(idx, ptr[r], ptr[r + 1], v, red, u);
     if (threadIdx.x == 0) out[r] = t;
 }
 
