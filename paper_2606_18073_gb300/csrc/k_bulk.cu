@@ -14,7 +14,9 @@
 //   A W columns replace a second pass over A (A (W y) = (A W) y).  In the final call of an
 //   iteration the kernel also forms ||x_k - x_{k-1}||^2, ||x_{k-1}||^2 (eq. RC) and
 //   ||x_k - x_true||^2 (RRE, Sec. 4) and the last CTA to finish reduces the CTA partials in
-//   a fixed order and records RC_k / RRE_k (no atomics on floating-point data).
+//   a fixed order and records RC_k / RRE_k (no atomics on floating-point data).  At 256^2 latency bounds
+//   it, and the statistics are a third of that: 24 us with all CTAs and one thread for both quotients,
+//   about 20 now (launch included).
 #include <math.h>
 
 #include "sgks_internal.cuh"

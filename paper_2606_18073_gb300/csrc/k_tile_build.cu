@@ -479,9 +479,9 @@ int build_tiles64(const sgks_reg* reg, const int32_t* rp, const int32_t* ci, con
     }
     TiledA a{};
     TiledT t{};
-    int rc = build_tiles_t(trp, tci, tval, m, n, nnz, reg->nx, reg->ny, nt, tile_ty(B), tile_stage(B), t, allocs, st, why);
+    int rc = build_tiles_t(trp, tci, tval, m, n, nnz, reg->nx, reg->ny, nt, tile_ty(B), tile_stage(std::min(B, 8)), t, allocs, st, why);
     if (rc != SGKS_OK || !t.ntiles) return rc;
-    const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, B / kTileInst);
+    const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, B / kTileInst);   // as measured, also for four instances per CTA
     rc = build_tiles(rp, ci, val, m, n, nnz, reg->nx, reg->ny, nt, ctas < 4 * 152 ? 16 : 32, 16, a, allocs, st, why);
     if (rc != SGKS_OK || !a.ntiles || a.nseg * 4 > nnz) return rc;
     T = a;

@@ -4,14 +4,15 @@
 // Bound: an FP64 warp instruction takes its quarter of the SM for 64 clocks on GB300, 0.63 T FMA/s for the
 // chip: 95 us per pass of the 512^2 CT operator (60 M entries), 71 us for its bytes.  The row kernels took 302
 // and 285 us there for a single vector (a scattered L2 load per entry), 171 and 413 us for 16 instances of the
-// 256^2 tomography problem (floor 60).  Here the gathered side lies in shared memory, entries come in order, and
+// 256^2 tomography problem (floor 60).  Now 147 (127 + 20 for the partials' sums; the FP64 pipe of the first
+// kernel is 90 % busy) and 151 us, 119 and 180 us for the 16 instances.  Here the gathered side lies in shared memory, entries come in order, and
 // the FP64 pipe does nothing but the multiply-adds:
 // - segments of a tile are sorted by length, so that the lanes of a warp run equally long;
 // - a conversion from FP32 costs as much as a multiply-add, so a value's bits are only moved into place: as
 //   a double they are a 2^-896 exactly (FP32 subnormals included).  Staged values are multiplied by 2^448
 //   and sums by 2^448 once each, which leaves products between 2^-574 and 2^576 exact; outside of
 //   that the solver's squared norms have under- or overflowed before.  An operator with infinite or NaN values
-//   keeps the row kernels (build_tiles64);
+//   keeps the row kernels (build_tiles64), and so does one with fewer than 2^20 entries;
 // - with several instances a lane takes up to four of them, for one entry load and one set of bit moves.
 #include <algorithm>
 
@@ -223,10 +224,14 @@ static cudaError_t apply64_ic(const TiledA& T, const TileVec64& W, double* part,
     return launch_pdl(k, (unsigned)(ctas * split), kThreads, smem, st, T, W, split, part);
 }
 
-cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, int lanes, double* part,
+cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, bool alone, double* part,
                                 const DevL& L, double* lw, cudaStream_t st) {
     cudaError_t e;
-    switch (std::min(W.B, kTileInst)) {
+    // Four instances per CTA give every lane a segment of its own, and a warp waits for one staged tile less
+    // often; the entries, read once per CTA, stay cheap next to the multiply-adds: 16 instances of 256^2
+    // take 147 us with 16 per CTA, 142 with 8, 119 with 4.  Several groups side by side hide those waits
+    // themselves and gain from fewer reads (groups of 8, 2 and 1, 243^2: 8.2 against 8.6 ms per solve).
+    switch (std::min(W.B, alone ? 4 : kTileInst)) {
         case 1: e = apply64_ic<1>(T, W, part, st); break;
         case 2: e = apply64_ic<2>(T, W, part, st); break;
         case 4: e = apply64_ic<4>(T, W, part, st); break;
@@ -234,6 +239,7 @@ cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileV
         default: e = apply64_ic<16>(T, W, part, st); break;
     }
     if (e != cudaSuccess) return e;
+    const int lanes = seg_lanes(W.B, alone);
     const int nbu = (int)std::max<int64_t>(1, std::min<int64_t>((m * W.B * lanes + kThreads - 1) / kThreads, 8 * 152));
     const int nbl = lw ? (int)std::max<int64_t>(1, std::min<int64_t>((L.p + kThreads - 1) / kThreads, 8 * 152)) : 0;
     return launch_pdl(kd_seg_reduce, nbu + nbl, kThreads, 0, st, T, U, m, part, lanes, nbu, L, W, lw);
@@ -258,12 +264,13 @@ static cudaError_t gradient64_ic(const TiledT& T, const TileVec64& E, const Tile
 
 cudaError_t launch64_tile_gradient(const TiledT& T, const TileVec64& E, const TileVec64& O, DevScalars* sc, const DevL& L,
                                    const double* x, const double* lam, double lam1, cudaStream_t st) {
-    switch (std::min(E.B, kTileInst)) {
+    // at most eight instances per CTA: 16 instances of 256^2 take 189 us with 16 per CTA (512 rays a stage),
+    // 180 with 8 (1024 rays), 196 with 4 (2048)
+    switch (std::min(E.B, 8)) {
         case 1: return gradient64_ic<1>(T, E, O, sc, L, x, lam, lam1, st);
         case 2: return gradient64_ic<2>(T, E, O, sc, L, x, lam, lam1, st);
         case 4: return gradient64_ic<4>(T, E, O, sc, L, x, lam, lam1, st);
-        case 8: return gradient64_ic<8>(T, E, O, sc, L, x, lam, lam1, st);
-        default: return gradient64_ty<16, 8>(T, E, O, sc, L, x, lam, lam1, st);
+        default: return gradient64_ic<8>(T, E, O, sc, L, x, lam, lam1, st);
     }
 }
 

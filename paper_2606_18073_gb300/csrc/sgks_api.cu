@@ -132,7 +132,7 @@ struct Engine : EngineBase {
     cudaError_t op_apply(int which, const T* in, T* out) {
         if constexpr (std::is_same<T, double>::value) {
             if (Ta.ntiles && which == SGKS_APPLY_A)
-                return launch64_tile_apply(Ta, plain64(in), plain64(out), D.m, seg_lanes(1, true), tpart, L, nullptr, st);
+                return launch64_tile_apply(Ta, plain64(in), plain64(out), D.m, true, tpart, L, nullptr, st);
             if (Ta.ntiles && which == SGKS_APPLY_AT)
                 return launch64_tile_gradient(Tt, plain64(in), plain64(out), nullptr, L, nullptr, nullptr, 0.0, st);
         }
@@ -142,7 +142,7 @@ struct Engine : EngineBase {
     cudaError_t op_new_column() {
         if constexpr (std::is_same<T, double>::value)
             if (Ta.ntiles)
-                return launch64_tile_apply(Ta, column64(B.W, D.n), column64(B.AW, D.m), D.m, seg_lanes(1, true), tpart, L, B.tmp_p, st);
+                return launch64_tile_apply(Ta, column64(B.W, D.n), column64(B.AW, D.m), D.m, true, tpart, L, B.tmp_p, st);
         return launch_apply_new_column<T, V>(D, A, L, B, S, st);
     }
     cudaError_t op_gradient_append() {

@@ -125,7 +125,7 @@ struct Group : GroupBase {
     cudaError_t op_apply(int which, const T* in, T* out) {
         if constexpr (sizeof(T) == 8) {
             if (Ta.ntiles && which == SGKS_APPLY_A)
-                return launch64_tile_apply(Ta, plain64(in), plain64(out), D.m, seg_lanes(D.B, D.alone), tpart, L, nullptr, st);
+                return launch64_tile_apply(Ta, plain64(in), plain64(out), D.m, D.alone, tpart, L, nullptr, st);
             if (Ta.ntiles)
                 return launch64_tile_gradient(Tt, plain64(in), plain64(out), nullptr, L, nullptr, nullptr, 0.0, st);
         }
@@ -134,7 +134,7 @@ struct Group : GroupBase {
     cudaError_t op_new_column() {
         if constexpr (sizeof(T) == 8)
             if (Ta.ntiles) {
-                const cudaError_t e = launch64_tile_apply(Ta, column64(X.W, D.n), column64(X.AW, D.m), D.m, seg_lanes(D.B, D.alone), tpart, L, nullptr, st);
+                const cudaError_t e = launch64_tile_apply(Ta, column64(X.W, D.n), column64(X.AW, D.m), D.m, D.alone, tpart, L, nullptr, st);
                 return e == cudaSuccess ? launchb_apply_column<T, V>(D, A, L, X, S, st, false) : e;
             }
         return launchb_apply_column<T, V>(D, A, L, X, S, st);

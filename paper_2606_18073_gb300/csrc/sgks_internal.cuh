@@ -1055,7 +1055,7 @@ struct TileVec64 {
     }
 };
 // U = A W through the tiles (part: npart x B doubles); lw (single handle): L w too, else null
-cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, int lanes, double* part,
+cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileVec64& U, int64_t m, bool alone, double* part,
                                 const DevL& L, double* lw, cudaStream_t st);
 // O = A^T E + lambda L^T L x (x null: A^T E); lambda per instance (lam) or one (lam1).  O without scalars but
 // sc given: instances that have stopped are left out.
