@@ -751,18 +751,19 @@ def main_batch(args):
         dist.destroy_process_group()
 
 
-BATCH_KERNEL_NAMES = {"apply_column": "kbx_csr_apply", "gradient_append": "kbx_csr_gradient",
-                      "combine": "kbx_combine_tma", "sketch_gather": "kbx_sketch_gather",
-                      "qr_append": "k_qr_append", "stacked_solve": "k_stacked_solve",
-                      "sketch_l": "kbx_sketch_l_chunks+kbx_sketch_l_reduce"}
+BATCH_KERNEL_NAMES = {"combine": "kb_combine_tma", "sketch_gather": "kb_sketch_gather",
+                      "apply_column": "kd_tile_apply+kd_seg_reduce", "gradient_append": "kd_tile_gradient",
+                      "qr_append": "k_qr_append", "stacked_solve": "k_stacked_solve"}
+# the compensated forms: both sketches by column chunks ("sketch_l"), their partials' sums ("sketch_gather")
+BATCH_KERNEL_NAMES_X = {"combine": "kbx_combine_tma", "sketch_l": "kbx_sketch_chunks", "sketch_gather": "kbx_sketch_reduce",
+                        "apply_column": "kbx_tile_apply+kbx_seg_reduce", "gradient_append": "kbx_tile_gradient"}
 
 
 def batch_kernel_name(kind, prec):
-    """The kernels behind a profile class of the batched CT workload (A w runs through pixel tiles
-    in the compensated forms)."""
-    if kind == "apply_column" and prec in ("ff", "fp32"):
-        return "kbx_tile_apply+kbx_seg_reduce"
-    return BATCH_KERNEL_NAMES.get(kind, kind)
+    """The kernels behind a profile class of the batched CT workload (the operator passes run through
+    pixel tiles)."""
+    name = BATCH_KERNEL_NAMES_X.get(kind) if prec in ("ff", "fp32") else None
+    return name or BATCH_KERNEL_NAMES.get(kind, kind)
 
 
 def traffic_record_batch(kernel, prec):

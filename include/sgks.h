@@ -140,11 +140,10 @@ typedef struct sgks_options {
                              bit 3 (SGKS_FLAG_AUTOTUNE, batches only): after the setup, time the
                              candidate tile choices of each group on its own data and keep the
                              fastest (bulk-copy slice 8 or 16 KB; lanes per CSR row of A and A^T;
-                             instances per CTA of the tiled forward pass, the default or twice it),
+                             instances per CTA of the tiled forward pass, the default or half of it),
                              a candidate replacing the default only when at least 5% faster;
                              results are cached per shape for the process.  Without it the
-                             defaults are used (16 KB, 8, 8; 8 float-float or 16 FP32 instances
-                             per tile CTA) and results are reproducible from run to run; the slice
+                             defaults are used (16 KB, 8, 8; 16 instances per tile CTA) and results are reproducible from run to run; the slice
                              and the tile instances keep every sum's order, the lanes per CSR row
                              change it (at the level of rounding).
                              bit 4 (SGKS_FLAG_NO_TILES, batches only): the compensated forms

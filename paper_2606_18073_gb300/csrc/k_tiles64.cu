@@ -5,8 +5,8 @@
 // chip: 95 us per pass of the 512^2 CT operator (60 M entries), 71 us for its bytes.  The row kernels took 302
 // and 285 us there for a single vector (a scattered L2 load per entry), 171 and 413 us for 16 instances of the
 // 256^2 tomography problem (floor 60).  Now 147 (127 + 20 for the partials' sums; the FP64 pipe of the first
-// kernel is 90 % busy) and 151 us, 119 and 180 us for the 16 instances.  Here the gathered side lies in shared memory, entries come in order, and
-// the FP64 pipe does nothing but the multiply-adds:
+// kernel is 90 % busy) and 151 us, 119 and 180 us for the 16 instances.  Here the gathered side lies in shared
+// memory, entries come in order, and the FP64 pipe does nothing but the multiply-adds:
 // - segments of a tile are sorted by length, so that the lanes of a warp run equally long;
 // - a conversion from FP32 costs as much as a multiply-add, so a value's bits are only moved into place: as
 //   a double they are a 2^-896 exactly (FP32 subnormals included).  Staged values are multiplied by 2^448
