@@ -573,6 +573,7 @@ __global__ void __launch_bounds__(kThreads) kbx_gradient(BDims D, DevA<float, fl
 // lane sums go to FP64 in shared memory, one partial per CTA and instance.
 template <typename TW, int NB>
 __global__ void __launch_bounds__(kThreads, 2) kbx_wtr(BDims D, BBulkX<TW> X, BSmall S, const float2* __restrict__ r) {
+    pdl_wait();
     pdl_trigger();   // the refinement solve loads X meanwhile
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_dlive;

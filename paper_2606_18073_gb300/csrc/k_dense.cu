@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(kThreads) k_dense_pair(Dims D, const TA* __res
                                                          Small S, const double* __restrict__ SA,
                                                          const double* __restrict__ SL, DensePlan PA, DensePlan PL,
                                                          DenseWork K) {
+    pdl_wait();
     pdl_trigger();   // the QR append loads its earlier columns meanwhile
     if (S.sc->stop) return;
     const int d = S.sc->d;

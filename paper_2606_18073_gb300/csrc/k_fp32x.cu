@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(kThreads) kx_gradient_append(Dims D, DevA<floa
 template <bool WARPA>
 __global__ void __cluster_dims__(kXCluster, 1, 1) __launch_bounds__(kThreads)
     kx_gradient_refine(Dims D, DevA<float, float> A, DevL L, BulkX B, Small S) {
+    pdl_wait();
     pdl_trigger();   // the refinement solve loads X meanwhile
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* gacc = reinterpret_cast<double*>(smem_raw);       // [dmax]

@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(kSketchThreads<IC>, IC >= 16 ? 2 : 4)
 template <int NB>
 __global__ void __launch_bounds__(kThreads) kbx_sketch_reduce(BDims D, SketchChunks K, BSmall S,
                                                               const float2* __restrict__ part, double* vec_out) {
+    pdl_wait();
     pdl_trigger();   // the QR append loads its earlier columns meanwhile
     __shared__ double red[NB][kThreads];
     const int B = D.B, H = B / NB, strands = kThreads / H;

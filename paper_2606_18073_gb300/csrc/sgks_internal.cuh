@@ -147,19 +147,25 @@ __device__ __forceinline__ bool mbar_wait_n(uint64_t* bar, uint32_t parity, int 
 
 // ----------------------------------------------------- programmatic dependent launch (PDL)
 // The kernels of one iteration follow each other on one stream.  Launched with the
-// programmatic-serialization attribute (launch_pdl), a kernel is launched as soon as every CTA of
-// the kernel before it has exited, without waiting for that grid's completion to be processed;
-// its CTAs then wait in pdl_wait until the predecessor's writes are visible.  This overlaps each
-// kernel's launch and CTA start-up with the end of its predecessor.  (Signalling earlier from
-// inside the predecessor, with griddepcontrol.launch_dependents at its start, was measured
-// slower: the waiting CTAs then hold SM resources through the whole predecessor.)  Every kernel
-// launched with launch_pdl calls pdl_wait before it touches global memory; for a kernel launched
-// without the attribute the call does nothing.
+// programmatic-serialization attribute (launch_pdl), a kernel starts as soon as every CTA of the
+// kernel before it has exited or called pdl_trigger, without waiting for that grid's completion
+// to be processed; its CTAs then wait in pdl_wait until the predecessor has finished and its writes
+// are visible.  This overlaps each kernel's launch and CTA start-up with its predecessor.  Rules:
+// - every kernel launched with launch_pdl calls pdl_wait, in every CTA, before it writes global memory
+//   and before it reads what its predecessor or any kernel still running may write;
+// - a kernel calls pdl_trigger only after its own pdl_wait, also where it is launched plainly today (the
+//   wait then does nothing).  So when a kernel starts, its predecessor has passed its wait, and everything
+//   before the predecessor is complete and visible;
+// - what may be read before pdl_wait is therefore what neither the predecessor nor this kernel writes: data
+//   fixed since the handle's creation (sketch entries, k_sketch.cu) and the factors and scalars that
+//   earlier kernels left (k_small2.cu: d, Q_A, Q_L, Q_T, X, z, d_A and S_A b, which the sketch, gradient
+//   and refinement kernels in front of it only read).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Lets the next kernel's CTAs start while this one still runs (its pdl_wait returns when this one has
-// finished).  Used where the next kernel is one of the small FP64 cluster kernels: 16 to 64 CTAs that fit
-// beside the others and have an earlier state to load (k_small2.cu).
+// finished); after pdl_wait, see above.  Used where the next kernel is one of the small FP64 cluster
+// kernels: 16 to 64 CTAs that fit beside the others and have an earlier state to load (k_small2.cu).  Before
+// a large kernel it does not pay: the waiting CTAs hold SM resources through the whole predecessor.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // SGKS_PDL=0 in the environment launches plainly (for comparison); default on.
