@@ -876,7 +876,7 @@ cudaError_t launchb_combine(const BDims& D, const BBulk<T>& X, const BSmall& S, 
     if (D.tma) {
         const size_t smem = batch_combine_tma_smem(sizeof(T), D.slice_kb);
         auto k = D.slice_kb == 8 ? kb_combine_tma<T, 6, 8192> : kb_combine_tma<T, 4, 16384>;
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
         k<<<D.nb_combine, kThreads, smem, st>>>(D, X, S, mode);
         return cudaGetLastError();
@@ -906,10 +906,8 @@ template <typename T, int NB>
 static cudaError_t wtr_nb(const BDims& D, const BBulk<T>& X, const BSmall& S, const T* r, cudaStream_t st) {
     const size_t smem = batch_refine_smem(D.dmax, D.B, sizeof(T));
     auto k = kb_wtr<T, NB>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
     k<<<D.nb_refine, kThreads, smem, st>>>(D, X, S, r);
     return cudaGetLastError();
 }

@@ -721,7 +721,7 @@ static int xcomb_per_sm(int slice_kb) {
     auto k = slice_kb == 8 ? kbx_combine_tma<TW, 6, 8192> : kbx_combine_tma<TW, 4, 16384>;
     const size_t smem = batchx_combine_smem(sizeof(TW), slice_kb);
     int nb = 0;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_smem(k, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kCombThreads, smem) != cudaSuccess || nb < 1) {
         (void)cudaGetLastError();
         nb = 1;
@@ -744,7 +744,7 @@ cudaError_t launchbx_combine(const BDims& D, const BBulkX<TW>& X, const BSmall& 
     if (D.tma) {
         const size_t smem = batchx_combine_smem(sizeof(TW), D.slice_kb);
         auto k = D.slice_kb == 8 ? kbx_combine_tma<TW, 6, 8192> : kbx_combine_tma<TW, 4, 16384>;
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
         k<<<D.nb_combine, kCombThreads, smem, st>>>(D, X, S, mode);
         return cudaGetLastError();
@@ -773,10 +773,8 @@ template <typename TW, int NB>
 static cudaError_t x_wtr_nb(const BDims& D, const BBulkX<TW>& X, const BSmall& S, const float2* r, cudaStream_t st) {
     const size_t smem = (size_t)D.dmax * D.B * sizeof(double) + 1024 * sizeof(float2);
     auto k = kbx_wtr<TW, NB>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
     k<<<D.nb_refine, kThreads, smem, st>>>(D, X, S, r);
     return cudaGetLastError();
 }

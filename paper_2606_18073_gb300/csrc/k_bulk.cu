@@ -188,12 +188,14 @@ cudaError_t launch_gradient(const Dims& D, const DevA<T, V>& A, const DevL& L, c
     const size_t smem = (size_t)D.dmax * sizeof(double) + kThreads * sizeof(T) + 128 * sizeof(T);
     if (warpa) {
         auto k = k_gradient_refine<T, V, true>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(k, smem);
+        if (e != cudaSuccess) return e;
         carveout_once((const void*)k);
         return launch_pdl(k, D.nbG, kThreads, smem, st, D, A, L, B, S);
     } else {
         auto k = k_gradient_refine<T, V, false>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(k, smem);
+        if (e != cudaSuccess) return e;
         carveout_once((const void*)k);
         return launch_pdl(k, D.nbG, kThreads, smem, st, D, A, L, B, S);
     }
@@ -359,10 +361,8 @@ template <typename T, int VW>
 static cudaError_t combine_vw(const Dims& D, const Bulk<T>& B, const Small& S, int mode, cudaStream_t st) {
     const size_t smem = (size_t)(D.dmax + kCombCols) * sizeof(T);
     auto k = k_combine<T, VW>;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
     carveout_once((const void*)k);
     const int64_t per = (int64_t)kThreads * VW;
     const int nbx = (int)((D.n + per - 1) / per), nbe = (int)((D.m + per - 1) / per);

@@ -305,18 +305,12 @@ static size_t conv_stage_bytes(int rt, int nx, int K) {
     return (size_t)conv_stage_rows(rt, nx, K) * (nx + 2 * kPad) * sizeof(T);
 }
 
-template <typename Kern>
-static cudaError_t smem_attr(Kern k, size_t smem) {
-    if (smem > 48 * 1024) return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return cudaSuccess;
-}
-
 template <typename T, typename V, int K>
 static cudaError_t append_k(const Dims& D, const DevA<T, V>& A, const DevL& L, const Bulk<T>& B, const Small& S,
                             cudaStream_t st) {
     auto k = k_gradient_append_conv<T, V, K>;
     const size_t smem = conv_stage_bytes<T>(kConvTile, A.nx, K);
-    cudaError_t e = smem_attr(k, smem);
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(k, conv_blocks(D.n), kThreads, smem, st, D, A, L, B, S);
 }
@@ -326,7 +320,7 @@ static cudaError_t apply_k(const Dims& D, const DevA<T, V>& A, const DevL& L, co
                            cudaStream_t st) {
     auto k = k_apply_column_conv<T, V, K>;
     const size_t smem = conv_stage_bytes<T>(kConvTile, A.nx, K);
-    cudaError_t e = smem_attr(k, smem);
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     const int nbc = conv_blocks(D.m);
     int64_t nbl = (D.p + kThreads - 1) / kThreads;
@@ -342,7 +336,7 @@ static cudaError_t refine_k(const Dims& D, const DevA<T, V>& A, const DevL& L, c
     auto k = k_gradient_refine2<T, V, MODE, K, CB>;
     size_t smem = (size_t)((D.dmax + 1) & ~1) * sizeof(double) + kThreads * sizeof(T);
     if (MODE == 2) smem += conv_stage_bytes<T>(kThreads, A.nx, K);
-    cudaError_t e = smem_attr(k, smem);
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     carveout_once((const void*)k);
     return launch_pdl(k, D.nbG, kThreads, smem, st, D, A, L, B, S);

@@ -427,11 +427,6 @@ cudaError_t launchx_to_float(const float2* in, float* out, int64_t n, cudaStream
 }
 
 // ------------------------------------------------------------------------------ launchers
-template <typename K>
-static void maybe_smem(K k, size_t bytes) {
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 static int x_apply_blocks(const Dims& D) {
     const int64_t slabs = (D.m + 31) / 32 + (D.p + 31) / 32;
     int64_t blocks = (slabs + kWarps - 1) / kWarps;
@@ -451,8 +446,7 @@ cudaError_t launchx_sketch_column(const Dims& D, const DevA<float, float>& A, co
 }
 
 cudaError_t launchx_combine(const Dims& D, const BulkX& B, const Small& S, int mode, cudaStream_t st) {
-    const size_t smem = (size_t)D.dmax * sizeof(float2);
-    maybe_smem(kx_combine, smem);
+    const size_t smem = (size_t)D.dmax * sizeof(float2);   // 16 KB at most (d_max <= kMaxS)
     carveout_once((const void*)kx_combine);
     kx_combine<<<D.nbX + D.nbE, kThreads, smem, st>>>(D, B, S, mode);
     return cudaGetLastError();
@@ -469,8 +463,8 @@ cudaError_t launchx_gradient(const Dims& D, const DevA<float, float>& A, const D
         return cudaGetLastError();
     }
     const size_t smem = (size_t)D.dmax * sizeof(double) + kThreads * sizeof(float2) + 128 * sizeof(float);
-    if (warpa) { maybe_smem(kx_gradient_refine<true>, smem); carveout_once((const void*)kx_gradient_refine<true>); kx_gradient_refine<true><<<D.nbG, kThreads, smem, st>>>(D, A, L, B, S); }
-    else { maybe_smem(kx_gradient_refine<false>, smem); carveout_once((const void*)kx_gradient_refine<false>); kx_gradient_refine<false><<<D.nbG, kThreads, smem, st>>>(D, A, L, B, S); }
+    if (warpa) { carveout_once((const void*)kx_gradient_refine<true>); kx_gradient_refine<true><<<D.nbG, kThreads, smem, st>>>(D, A, L, B, S); }
+    else { carveout_once((const void*)kx_gradient_refine<false>); kx_gradient_refine<false><<<D.nbG, kThreads, smem, st>>>(D, A, L, B, S); }
     return cudaGetLastError();
 }
 

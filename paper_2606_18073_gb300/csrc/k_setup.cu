@@ -38,6 +38,21 @@ void carveout_once(const void* kernel) {
         cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pref);
 }
 
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+    if (bytes <= 8 * 1024) return cudaSuccess;   // no kernel here has 40 KB of its own
+    cudaFuncAttributes at;
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+    if (e != cudaSuccess || bytes + at.sharedSizeBytes <= 48 * 1024) return e;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    const int most = optin - (int)at.sharedSizeBytes;
+    if (bytes > (size_t)(most > 0 ? most : 0)) return cudaErrorInvalidValue;
+    if (at.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // ---------------------------------------------------------------------------- applies
 template <typename T, typename V, bool WARPA, int LPR = 32, bool SL = false>
 __global__ void __launch_bounds__(kThreads) k_apply(DevA<T, V> A, DevL L, int which, const T* __restrict__ in,

@@ -231,10 +231,8 @@ static cudaError_t sketch_chunks_ic(const BDims& D, const DevL& L, const BBulkX<
                                     const BSmall& S, float2* part, bool a_only, cudaStream_t st) {
     const size_t smem = (size_t)(K.C + 1) * IC * sizeof(float2);
     auto k = kbx_sketch_chunks<TW, IC>;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
     const int64_t chunks = a_only ? K.nA : K.nA + K.nL;
     k<<<(unsigned)(chunks * (D.B / IC)), kSketchThreads<IC>, smem, st>>>(D, L, X, K, S, part);
     return cudaGetLastError();

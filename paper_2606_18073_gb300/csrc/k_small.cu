@@ -310,10 +310,8 @@ static cudaError_t config_cs(int s, int dm) {
         e = cudaFuncSetAttribute(k_refine_solve<CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
-    e = cudaFuncSetAttribute(k_append_solve<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)append_smem(s, dm, CS));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_refine_solve<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)refine_smem(dm));
+    e = allow_smem(k_append_solve<CS>, append_smem(s, dm, CS));
+    if (e == cudaSuccess) e = allow_smem(k_refine_solve<CS>, refine_smem(dm));
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CS);

@@ -529,12 +529,8 @@ static cudaError_t config2(int s, int dm, size_t limit) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_refine_solve2<CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
-    e = cudaFuncSetAttribute(k_qr_append<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_stacked_solve<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_refine_solve2<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(2 * sizeof(double) * (size_t)dm));
+    e = allow_smem(k_qr_append<CS>, qr_append_smem(s, dm, CS, halves(qr_append_smem(s, dm, CS, 2))));
+    if (e == cudaSuccess) e = allow_smem(k_stacked_solve<CS>, stacked_smem(dm, CS, halves(stacked_smem(dm, CS, 2))));
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * CS);

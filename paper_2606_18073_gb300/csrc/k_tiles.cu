@@ -346,17 +346,12 @@ __global__ void __launch_bounds__(GradShape<IC, TY>::threads, IC >= 16 ? 3 : 102
 // ------------------------------------------------------------------------------ launchers
 int tile_instances(const BDims& D) { return std::min(D.B, D.tile_ic > 0 ? D.tile_ic : kTileInst); }
 
-template <typename K>
-static cudaError_t tile_smem_limit(K k, size_t smem) {
-    return smem > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
-}
-
 template <typename TW, int IC>
 static cudaError_t tile_apply_ic(const BDims& D, const TiledA& T, const BBulkX<TW>& X, const BSmall& S, float2* part,
                                  cudaStream_t st) {
     const size_t smem = (size_t)(T.TX * T.TY + 1) * IC * sizeof(TW);
     auto k = kbx_tile_apply<TW, IC>;
-    cudaError_t e = tile_smem_limit(k, smem);
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     // A tile's segments go to `split` CTAs (each stages the tile) until there are eight rounds of CTAs:
     // with 4.5 rounds, 512^2 at 64 instances, the last one leaves a tenth of the chip's time unused.
@@ -391,7 +386,7 @@ static cudaError_t tile_gradient_ty(const BDims& D, const TiledT& T, const DevL&
                                     float2* out, cudaStream_t st) {
     const size_t smem = (size_t)(T.stage + 1) * IC * sizeof(float2);
     auto k = kbx_tile_gradient<TW, IC, TY>;
-    const cudaError_t e = tile_smem_limit(k, smem);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     k<<<(unsigned)((int64_t)T.ntiles * (D.B / IC)), GradShape<IC, TY>::threads, smem, st>>>(D, T, L, X, S, out);
     return cudaGetLastError();

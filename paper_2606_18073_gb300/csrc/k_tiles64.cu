@@ -206,16 +206,11 @@ __global__ void __launch_bounds__(kThreads, 3) kd_tile_gradient(TiledT T, TileVe
 }
 
 // ------------------------------------------------------------------------------ launchers
-template <typename K>
-static cudaError_t smem64(K k, size_t smem) {
-    return smem > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
-}
-
 template <int IC>
 static cudaError_t apply64_ic(const TiledA& T, const TileVec64& W, double* part, cudaStream_t st) {
     const size_t smem = (size_t)(T.TX * T.TY + 1) * IC * sizeof(double);
     auto k = kd_tile_apply<IC>;
-    const cudaError_t e = smem64(k, smem);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     // shares of a tile's segments until there are four rounds of CTAs, with four segments or more per lane
     const int64_t ctas = (int64_t)T.ntiles * (W.B / IC);
@@ -250,7 +245,7 @@ static cudaError_t gradient64_ty(const TiledT& T, const TileVec64& E, const Tile
                                  const double* x, const double* lam, double lam1, cudaStream_t st) {
     const size_t smem = (size_t)(T.stage + 1) * IC * sizeof(double);
     auto k = kd_tile_gradient<IC, TY>;
-    const cudaError_t e = smem64(k, smem);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(k, (unsigned)((int64_t)T.ntiles * (E.B / IC)), kThreads, smem, st, T, E, O, sc, L, x, lam, lam1);
 }

@@ -272,6 +272,15 @@ __device__ __forceinline__ double tree_sumd(const double* a, int stride = 1) {
 // preferred carveout on its first launch, so consecutive kernels need no SM reconfiguration.
 void carveout_once(const void* kernel);
 
+// More than 48 KB of shared memory has to be allowed kernel by kernel, and the limit belongs to the process: a
+// handle of another size, or another host thread between this call and the launch, changes it for everyone.  So it
+// is only ever raised, at once to all that a CTA can have.  cudaErrorInvalidValue where that is less than `bytes`.
+cudaError_t allow_smem(const void* kernel, size_t bytes);
+template <typename... KArgs>
+cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes) {
+    return allow_smem((const void*)kernel, bytes);
+}
+
 // SplitMix64 output function (Steele, Lea, Flood 2014).
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
