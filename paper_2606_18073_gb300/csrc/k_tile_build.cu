@@ -256,13 +256,12 @@ __global__ void k_group_pairs(const int32_t* __restrict__ used, int64_t groups, 
 
 unsigned grid_for(int64_t work) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(work, 16 * 152)); }
 
-// Device memory of one build on its stream; what is not handed over is freed at the end.
+// Device memory of one build on its stream; what is not handed over (keep) is freed at the end.
 struct Build {
     cudaStream_t st;
     cudaError_t e = cudaSuccess;
-    std::vector<void*> tmp;
-    std::vector<void*>* keep;
-    Build(cudaStream_t s, std::vector<void*>* k) : st(s), keep(k) {}
+    std::vector<void*> tmp, own;
+    explicit Build(cudaStream_t s) : st(s) {}
     template <typename P>
     P* temp(size_t count) {
         void* q = nullptr;
@@ -274,8 +273,12 @@ struct Build {
     P* held(size_t count) {
         void* q = nullptr;
         if (e == cudaSuccess) e = cudaMalloc(&q, count * sizeof(P) + 16);
-        if (e == cudaSuccess) keep->push_back(q);
+        if (e == cudaSuccess) own.push_back(q);
         return e == cudaSuccess ? (P*)q : nullptr;
+    }
+    void keep(std::vector<void*>& allocs) {
+        allocs.insert(allocs.end(), own.begin(), own.end());
+        own.clear();
     }
     void zero(void* p, size_t bytes) {
         if (e == cudaSuccess && bytes) e = cudaMemsetAsync(p, 0, bytes, st);
@@ -297,6 +300,7 @@ struct Build {
     }
     ~Build() {
         for (void* q : tmp) cudaFreeAsync(q, st);
+        for (void* q : own) cudaFree(q);   // waits for the kernels that use it
     }
 };
 
@@ -334,9 +338,14 @@ bool geometry(int64_t m, int64_t n, int nx, int ny, int nt, int TX, int TY, Geo*
     return tiles < ((int64_t)1 << 31);
 }
 
+// Without the memory for a layout the row kernels remain, which need none of it: no error.
 int failed(const Build& b, std::string* why) {
+    if (b.e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return SGKS_OK;
+    }
     *why = std::string("tiled operator: ") + cudaGetErrorString(b.e);
-    return b.e == cudaErrorMemoryAllocation ? SGKS_ERR_NOMEM : SGKS_ERR_CUDA;
+    return SGKS_ERR_CUDA;
 }
 
 int refused(std::string* why, const char* what) {
@@ -346,6 +355,29 @@ int refused(std::string* why, const char* what) {
 
 }  // namespace
 
+bool tile_room(std::vector<void*>& allocs) {
+    size_t room = 0, total = 0;
+    if (cudaMemGetInfo(&room, &total) == cudaSuccess && room >= kTileRoom) return true;
+    cudaGetLastError();
+    drop_tile_memory(allocs);
+    return false;
+}
+
+bool tile_memory(std::vector<void*>& allocs, void** p, size_t bytes) {
+    if (cudaMalloc(p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        drop_tile_memory(allocs);
+        return false;
+    }
+    allocs.push_back(*p);
+    return tile_room(allocs);
+}
+
+void drop_tile_memory(std::vector<void*>& allocs) {
+    for (void* q : allocs) cudaFree(q);
+    allocs.clear();
+}
+
 int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t m, int64_t n, int64_t nnz, int nx, int ny,
                 int nt, int TX, int TY, TiledA& T, std::vector<void*>& allocs, cudaStream_t st, std::string* why) {
     Geo g;
@@ -353,7 +385,7 @@ int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t 
         return refused(why, "geometry does not match the unknowns");
     const size_t nw = (size_t)g.ntiles * g.words;
     if (nw > kMaxWords) return SGKS_OK;
-    Build b(st, &allocs);
+    Build b(st);
     uint32_t* bits = b.temp<uint32_t>(nw);
     int32_t *before = b.temp<int32_t>(nw), *cnt = b.temp<int32_t>(g.ntiles), *rows = b.temp<int32_t>(g.words * 32);
     int32_t* err = b.temp<int32_t>(1);
@@ -370,7 +402,7 @@ int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t 
     if (herr[0]) return refused(why, "a row pointer or column index out of range");
     std::vector<int32_t> grp(hcnt), grp0, off;
     for (int32_t& v : grp) v = (v + 3) / 4;
-    if (!prefix(grp, &grp0) || grp0.back() >= (1 << 29)) return refused(why, "too many segments");
+    if (!prefix(grp, &grp0) || grp0.back() >= (1 << 29)) return SGKS_OK;
     const int64_t ngrp = grp0.back();
     int32_t* tile_grp = b.up(grp0);
     int32_t *len = b.temp<int32_t>(4 * ngrp), *pos = b.temp<int32_t>(4 * ngrp), *pairs = b.temp<int32_t>(ngrp);
@@ -380,10 +412,10 @@ int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t 
     k_seg_len<<<gr, kThreads, 0, st>>>(g, rp, ci, bits, before, tile_grp, len);
     k_seg_sort<<<g.ntiles, 32, 0, st>>>(tile_grp, cnt, len, pos, pairs);
     b.ran();
-    if (!prefix(b.down(pairs, ngrp), &off)) return refused(why, "too many entries");
+    if (!prefix(b.down(pairs, ngrp), &off)) return SGKS_OK;   // too many for 32-bit positions
     const int64_t npairs = (int64_t)off.back() + kTileAhead;
     int32_t *goff = b.up(off), *order = b.up(heavy_first(off, grp0, 1));
-    if (!prefix(b.down(rows, m), &off)) return refused(why, "too many segments");
+    if (!prefix(b.down(rows, m), &off)) return SGKS_OK;
     const int64_t nseg = off.back();
     int32_t *ray_ptr = b.up(off), *ray_seg = b.held<int32_t>(nseg);
     uint4* ent = b.held<uint4>(4 * npairs);
@@ -394,6 +426,7 @@ int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t 
                                         ray_seg);
     b.ran();
     if (b.e != cudaSuccess) return failed(b, why);
+    b.keep(allocs);
     T = TiledA{TX, TY, nx, ny, nt, g.ntx, g.nty, g.ntiles, 4 * ngrp, nseg, order, tile_grp, goff, ray_ptr, ray_seg, ent};
     return SGKS_OK;
 }
@@ -407,7 +440,7 @@ int build_tiles_t(const int32_t* trp, const int32_t* tci, const float* tval, int
         return refused(why, "geometry does not match the unknowns");
     const size_t nw = (size_t)g.ntiles * g.words;
     if (nw > kMaxWords) return SGKS_OK;
-    Build b(st, &allocs);
+    Build b(st);
     uint32_t* bits = b.temp<uint32_t>(nw);
     int32_t *before = b.temp<int32_t>(nw), *cnt = b.temp<int32_t>(g.ntiles), *err = b.temp<int32_t>(1);
     b.zero(bits, nw * 4);
@@ -449,6 +482,7 @@ int build_tiles_t(const int32_t* trp, const int32_t* tci, const float* tval, int
     k_pixel_entries<true><<<gc, kThreads, 0, st>>>(g, trp, tci, tval, bits, before, tile_stage, stage, used, goff, (uint32_t*)ent);
     b.ran();
     if (b.e != cudaSuccess) return failed(b, why);
+    b.keep(allocs);
     T = TiledT{TX, TY, nx, ny, nt, g.ntx, g.nty, g.ntiles, order, tile_stage, tile_ray, ray, goff, stage, ent};
     return SGKS_OK;
 }
@@ -467,7 +501,7 @@ int build_tiles64(const sgks_reg* reg, const int32_t* rp, const int32_t* ci, con
     const int nt = reg->kind == SGKS_REG_SPACETIME ? reg->nt : 1;
     if ((int64_t)reg->nx * reg->ny * nt != n) return SGKS_OK;
     {
-        Build b(st, &allocs);
+        Build b(st);
         int32_t* bad = b.temp<int32_t>(1);
         b.zero(bad, 4);
         if (b.e != cudaSuccess) return failed(b, why);
@@ -479,11 +513,13 @@ int build_tiles64(const sgks_reg* reg, const int32_t* rp, const int32_t* ci, con
     }
     TiledA a{};
     TiledT t{};
-    int rc = build_tiles_t(trp, tci, tval, m, n, nnz, reg->nx, reg->ny, nt, tile_ty(B), tile_stage(std::min(B, 8)), t, allocs, st, why);
+    Build both(st);   // holds the one layout until the other is there too
+    int rc = build_tiles_t(trp, tci, tval, m, n, nnz, reg->nx, reg->ny, nt, tile_ty(B), tile_stage(std::min(B, 8)), t, both.own, st, why);
     if (rc != SGKS_OK || !t.ntiles) return rc;
     const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, B / kTileInst);   // as measured, also for four instances per CTA
-    rc = build_tiles(rp, ci, val, m, n, nnz, reg->nx, reg->ny, nt, ctas < 4 * 152 ? 16 : 32, 16, a, allocs, st, why);
+    rc = build_tiles(rp, ci, val, m, n, nnz, reg->nx, reg->ny, nt, ctas < 4 * 152 ? 16 : 32, 16, a, both.own, st, why);
     if (rc != SGKS_OK || !a.ntiles || a.nseg * 4 > nnz) return rc;
+    both.keep(allocs);
     T = a;
     Tt = t;
     return SGKS_OK;

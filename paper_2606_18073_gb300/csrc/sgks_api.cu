@@ -77,7 +77,10 @@ struct EngineBase {
         return e;
     }
     bool gauss = false;
-    virtual ~EngineBase() {}
+    std::vector<void*> tile_allocs;   // layouts and partials of the tiled passes
+    virtual ~EngineBase() { drop_tile_memory(tile_allocs); }
+    // back to the row kernels (nothing in flight, no captured graph left): true if there were tiles
+    virtual bool drop_tiles() { return false; }
     virtual cudaError_t setup(const void* b) = 0;
     virtual cudaError_t step() = 0;
     // one launch of a streaming kernel class in the current state (sgks_time_class)
@@ -125,6 +128,15 @@ struct Engine : EngineBase {
     TiledA Ta{};
     TiledT Tt{};
     double* tpart = nullptr;        // [npart]
+
+    bool drop_tiles() override {
+        const bool had = Ta.ntiles != 0;
+        Ta = TiledA{};
+        Tt = TiledT{};
+        tpart = nullptr;
+        drop_tile_memory(tile_allocs);
+        return had;
+    }
 
     TileVec64 plain64(const T* v) const { return TileVec64{(const double*)v, 0, nullptr, 0, 1}; }
     TileVec64 column64(const T* v, int64_t rows) const { return TileVec64{(const double*)v, rows, S.sc, D.dmax, 1}; }
@@ -305,6 +317,7 @@ struct Engine : EngineBase {
 
     cudaError_t bw_prepare() {
         if (bw.Wb) return cudaSuccess;
+        const size_t held = allocs->size(), host_held = host_allocs->size();
         const size_t n = D.n, m = D.m, p = D.p, s = D.s, dm = D.dmax, ell = D.ell;
         cudaError_t e = cudaSuccess;
         auto A1 = [&](auto** ptr, size_t c) { if (e == cudaSuccess) e = bw_alloc(ptr, c); };
@@ -320,10 +333,6 @@ struct Engine : EngineBase {
                 e = cudaHostGetDevicePointer(&dp, hp, 0);
             }
             if (e == cudaSuccess) bw.Wb = (T*)dp;
-            if (e != cudaSuccess) {
-                bw.Wb = nullptr;
-                return e;
-            }
         } else {
             A1(&bw.Wb, dm * n);
         }
@@ -336,7 +345,11 @@ struct Engine : EngineBase {
             A1(&bw.w, dm); A1(&bw.dl, dm); A1(&bw.td, dm);
             A1(&bw.Ww, n); A1(&bw.HWw, n); A1(&bw.xp, n); A1(&bw.rho, n); A1(&bw.a1, n); A1(&bw.a2, n);
         }
-        if (e != cudaSuccess) bw.Wb = nullptr;
+        if (e != cudaSuccess) {   // keep no part of it
+            bw.Wb = nullptr;
+            for (; allocs->size() > held; allocs->pop_back()) cudaFree(allocs->back());
+            for (; host_allocs->size() > host_held; host_allocs->pop_back()) cudaFreeHost(host_allocs->back());
+        }
         return e;
     }
 
@@ -1235,16 +1248,6 @@ static int build_engine(sgks_handle* h, const sgks_op* op, const sgks_reg* reg, 
         std::string why;
         const int rc = prepare_operator<T, V>(op, E->A, h->allocs, E->d_err, h->st, &why);
         if (rc != SGKS_OK) return fail(h, rc, why);
-        if constexpr (std::is_same<T, double>::value && std::is_same<V, float>::value) {
-            if (op->kind == SGKS_OP_CSR) {
-                const int rt = build_tiles64(reg, E->A.rp, E->A.ci, E->A.val, E->A.trp, E->A.tci, E->A.tval, D.m, D.n, op->nnz, 1,
-                                             E->Ta, E->Tt, h->allocs, h->st, &why);
-                if (rt != SGKS_OK) return fail(h, rt, why);
-                if (E->Ta.ntiles) AL(E->tpart, E->Ta.npart);
-                if (e != cudaSuccess)
-                    return fail(h, SGKS_ERR_NOMEM, std::string("device allocation: ") + cudaGetErrorString(e));
-            }
-        }
         if (!gauss) {
             const int rs = prepare_sparse_sign(D.keyA, D.keyL, D.m, D.p, s, o.zeta, E->SK, h->allocs, E->d_err,
                                                h->st, &why);
@@ -1265,6 +1268,15 @@ static int build_engine(sgks_handle* h, const sgks_op* op, const sgks_reg* reg, 
         E->gSL = SL;
     }
 #undef AL
+    if constexpr (std::is_same<T, double>::value && std::is_same<V, float>::value)
+        if (op->kind == SGKS_OP_CSR) {   // after all else: the layouts are taken where there is room for them
+            std::string why;
+            const int rt = build_tiles64(reg, E->A.rp, E->A.ci, E->A.val, E->A.trp, E->A.tci, E->A.tval, D.m, D.n, op->nnz, 1,
+                                         E->Ta, E->Tt, E->tile_allocs, h->st, &why);
+            if (rt != SGKS_OK) return fail(h, rt, why);
+            if (E->Ta.ntiles && !tile_memory(E->tile_allocs, (void**)&E->tpart, sizeof(double) * (size_t)E->Ta.npart))
+                E->drop_tiles();
+        }
     return SGKS_OK;
 }
 
@@ -1445,6 +1457,17 @@ int sgks_backward(sgks_handle* h, const void* xbar, void* bbar, double* lambda_b
         return fail(h, SGKS_ERR_STATE, "the recorded solve did not complete its iterations cleanly");
     join_in(h);
     cudaError_t e = E->backward(xbar, bbar, lambda_bar, K);
+    if (e == cudaErrorMemoryAllocation) {   // the sweep's workspace comes before the tiled layouts
+        cudaGetLastError();
+        cudaStreamSynchronize(h->st);
+        if (E->drop_tiles()) {
+            if (h->gexec) cudaGraphExecDestroy(h->gexec);
+            if (h->graph) cudaGraphDestroy(h->graph);
+            h->gexec = nullptr;
+            h->graph = nullptr;
+            e = E->backward(xbar, bbar, lambda_bar, K);
+        }
+    }
     join_out(h);
     if (e != cudaSuccess) return cuda_fail(h, e, "sgks_backward");
     return SGKS_OK;

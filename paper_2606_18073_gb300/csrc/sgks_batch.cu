@@ -12,6 +12,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <new>
@@ -579,6 +580,7 @@ struct sgks_batch {
     cudaStream_t st = nullptr, user = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     std::vector<void*> allocs;
+    std::vector<std::function<int()>> tilers;   // at create: the tiled layouts, after all workspaces
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     int64_t graph_launches = 0;
@@ -795,6 +797,19 @@ std::vector<int> split_groups(size_t count, int bcap) {
     return out;
 }
 
+// The groups' partial sums of the tiled forward pass; empty, with everything in mem freed, when there is no layout
+// or no room for them.
+template <typename P, typename G>
+std::vector<P*> group_partials(std::vector<void*>& mem, const TiledA& Ta, const std::vector<G*>& groups) {
+    std::vector<P*> part;
+    for (size_t g = 0; Ta.ntiles && g < groups.size(); ++g) {
+        void* q = nullptr;
+        if (!tile_memory(mem, &q, sizeof(P) * (size_t)Ta.npart * groups[g]->D.B + 16)) return {};
+        part.push_back((P*)q);
+    }
+    return part;
+}
+
 template <typename T, typename V>
 int build_groups(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const std::vector<int>& inst,
                  const void* const* b, const double* lambdas, const void* const* x_true, int s, uint64_t seed,
@@ -814,14 +829,7 @@ int build_groups(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const st
     if (o.n_refine > 0 && batch_refine_smem(dmax, 1, sizeof(T)) > 200 * 1024)
         return bfail(h, SGKS_ERR_INVALID, "ell + max_iters too large for the batched refinement");
     const std::vector<int> sizes = split_groups(inst.size(), max_group_size(dmax, o.n_refine, sizeof(T)));
-    TiledA Ta{};
-    TiledT Tt{};
-    if constexpr (sizeof(T) == 8 && sizeof(V) == 4)
-        if (op->kind == SGKS_OP_CSR && !(o.flags & SGKS_FLAG_NO_TILES)) {
-            rc = build_tiles64(reg, A.rp, A.ci, A.val, A.trp, A.tci, A.tval, op->m, op->n, op->nnz, sizes[0], Ta, Tt, h->allocs,
-                               h->st, &why);
-            if (rc != SGKS_OK) return bfail(h, rc, why);
-        }
+    std::vector<Group<T, V>*> made;
     size_t pos = 0;
     for (const int B : sizes) {
         Group<T, V>* G = new (std::nothrow) Group<T, V>();
@@ -858,14 +866,31 @@ int build_groups(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const st
         BA(X.tp, pB);
         BA(X.tm, mB);
         if (o.n_refine > 0) BA(X.r, nB);
-        G->Ta = Ta;
-        G->Tt = Tt;
-        if (Ta.ntiles) BA(G->tpart, (size_t)Ta.npart * B);
 #undef BA
         if (e != cudaSuccess) return bfail(h, SGKS_ERR_NOMEM, std::string("device allocation: ") + cudaGetErrorString(e));
         e = cudaMemsetAsync(X.xs, 0, sizeof(T) * nB, h->st);
         if (e != cudaSuccess) return bcuda_fail(h, e, "batch workspace initialisation");
+        made.push_back(G);
     }
+    if constexpr (sizeof(T) == 8 && sizeof(V) == 4)
+        if (op->kind == SGKS_OP_CSR && !(o.flags & SGKS_FLAG_NO_TILES))
+            h->tilers.push_back([=] {
+                TiledA Ta{};
+                TiledT Tt{};
+                std::vector<void*> mem;
+                std::string why;
+                const int rc = build_tiles64(reg, A.rp, A.ci, A.val, A.trp, A.tci, A.tval, op->m, op->n, op->nnz, made[0]->D.B,
+                                             Ta, Tt, mem, h->st, &why);
+                if (rc != SGKS_OK) return bfail(h, rc, why);
+                std::vector<double*> part = group_partials<double>(mem, Ta, made);
+                for (size_t g = 0; g < part.size(); ++g) {
+                    made[g]->Ta = Ta;
+                    made[g]->Tt = Tt;
+                    made[g]->tpart = part[g];
+                }
+                h->allocs.insert(h->allocs.end(), mem.begin(), mem.end());
+                return SGKS_OK;
+            });
     return SGKS_OK;
 }
 
@@ -900,28 +925,14 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
     rc = prepare_sparse_sign(sketch_key_host_dev(seed, 0), sketch_key_host_dev(seed, 1), op->m, L.p, s, o.zeta, SK,
                              h->allocs, h->d_err, h->st, &why);
     if (rc != SGKS_OK) return bfail(h, rc, why);
-    // pixel tiles of a CSR operator on an image geometry (the regularizer's)
-    TiledA T{};
-    TiledT Tt{};
     const std::vector<int> sizes = split_groups(inst.size(), max_group_size(o.ell + o.max_iters, o.n_refine, sizeof(float2)));
     SketchChunks KC{};
     rc = build_sketch_chunks(SK, op->m, L.p, s, sizes[0], KC, h->allocs, h->st, &why);
     if (rc != SGKS_OK) return bfail(h, rc, why);
-    if (op->kind == SGKS_OP_CSR && !(o.flags & SGKS_FLAG_NO_TILES) &&
-        (reg->kind == SGKS_REG_GRAD2D || reg->kind == SGKS_REG_LAPLACE2D || reg->kind == SGKS_REG_SPACETIME)) {
-        const int nt = reg->kind == SGKS_REG_SPACETIME ? reg->nt : 1;
-        // 32 x 16 pixels leave a third fewer partial sums than 16 x 16; below four CTAs per SM the
-        // smaller tile spreads the pass over the chip instead
-        const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, sizes[0] / kTileInst);
-        rc = build_tiles(A.rp, A.ci, A.val, op->m, op->n, op->nnz, reg->nx, reg->ny, nt, ctas < 4 * 152 ? 16 : 32, 16, T,
-                         h->allocs, h->st, &why);
-        if (rc == SGKS_OK)
-            rc = build_tiles_t(A.trp, A.tci, A.tval, op->m, op->n, op->nnz, reg->nx, reg->ny, nt, tile_ty(sizes[0]), tile_stage(sizes[0]), Tt, h->allocs, h->st, &why);
-        if (rc != SGKS_OK) return bfail(h, rc, why);
-    }
     const int dmax = o.ell + o.max_iters;
     if (o.n_refine > 0 && batch_refine_smem(dmax, 1, sizeof(float2)) > 200 * 1024)
         return bfail(h, SGKS_ERR_INVALID, "ell + max_iters too large for the batched refinement");
+    std::vector<GroupX<TW>*> made;
     size_t pos = 0;
     for (const int B : sizes) {
         GroupX<TW>* G = new (std::nothrow) GroupX<TW>();
@@ -933,8 +944,6 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
         G->Ad = Ad;
         G->L = L;
         G->SK = SK;
-        G->T = T;
-        G->Tt = Tt;
         G->KC = KC;
         G->io_dt = io_dt;
         G->has_xt = x_true != nullptr;
@@ -964,7 +973,6 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
         BA(G->spart, (size_t)(KC.nA + KC.nL) * s * B);
         if (o.n_refine > 0) BA(X.r, nB);
         BA(lam2, B);
-        if (T.ntiles) BA(G->part, (size_t)T.npart * B);
         // the FP64 setup of W_0 (Krylov basis, CGS2): its ell columns, a temporary and b
         BA(G->Xd.W, (size_t)D.ell * nB);
         BA(G->Xd.tm, mB);
@@ -986,7 +994,37 @@ int build_groups_x(sgks_batch* h, const sgks_op* op, const sgks_reg* reg, const 
         if (e == cudaSuccess) e = cudaMemsetAsync(X.xs, 0, sizeof(float2) * nB, h->st);
         if (e == cudaSuccess && G->zlam) e = cudaMemsetAsync(G->zlam, 0, sizeof(float2) * B, h->st);
         if (e != cudaSuccess) return bcuda_fail(h, e, "batch workspace initialisation");
+        made.push_back(G);
     }
+    // pixel tiles of a CSR operator on an image geometry (the regularizer's)
+    if (op->kind == SGKS_OP_CSR && !(o.flags & SGKS_FLAG_NO_TILES) &&
+        (reg->kind == SGKS_REG_GRAD2D || reg->kind == SGKS_REG_LAPLACE2D || reg->kind == SGKS_REG_SPACETIME))
+        h->tilers.push_back([=] {
+            const int nt = reg->kind == SGKS_REG_SPACETIME ? reg->nt : 1, Bmax = made[0]->D.B;
+            // 32 x 16 pixels leave a third fewer partial sums than 16 x 16; below four CTAs per SM the
+            // smaller tile spreads the pass over the chip instead
+            const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, Bmax / kTileInst);
+            TiledA T{};
+            TiledT Tt{};
+            std::vector<void*> mem, mem_t;
+            std::string why;
+            int rc = build_tiles(A.rp, A.ci, A.val, op->m, op->n, op->nnz, reg->nx, reg->ny, nt, ctas < 4 * 152 ? 16 : 32, 16,
+                                 T, mem, h->st, &why);
+            if (rc != SGKS_OK) return bfail(h, rc, why);
+            std::vector<float2*> part = group_partials<float2>(mem, T, made);
+            for (size_t g = 0; g < part.size(); ++g) {
+                made[g]->T = T;
+                made[g]->part = part[g];
+            }
+            h->allocs.insert(h->allocs.end(), mem.begin(), mem.end());
+            rc = build_tiles_t(A.trp, A.tci, A.tval, op->m, op->n, op->nnz, reg->nx, reg->ny, nt, tile_ty(Bmax),
+                               tile_stage(Bmax), Tt, mem_t, h->st, &why);
+            if (rc != SGKS_OK) return bfail(h, rc, why);
+            if (!Tt.ntiles || !tile_room(mem_t)) return SGKS_OK;
+            for (GroupX<TW>* G : made) G->Tt = Tt;
+            h->allocs.insert(h->allocs.end(), mem_t.begin(), mem_t.end());
+            return SGKS_OK;
+        });
     return SGKS_OK;
 }
 
@@ -1117,6 +1155,8 @@ int sgks_batch_create(sgks_batch** hp, int32_t count, const sgks_op* A, const sg
             rc = build_groups<double, float>(h, op, reg, members[k], b, lambdas, x_true, sketch_rows, seed, o,
                                              cluster2);
     }
+    for (size_t k = 0; k < h->tilers.size() && rc == SGKS_OK; ++k) rc = h->tilers[k]();
+    h->tilers.clear();
     for (GroupBase* g : h->groups) g->D.alone = h->groups.size() == 1;
     if (rc == SGKS_OK && h->groups.size() > 1) {
         for (size_t g = 0; g < h->groups.size() && e == cudaSuccess; ++g) {

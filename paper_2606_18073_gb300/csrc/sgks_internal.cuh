@@ -1052,6 +1052,15 @@ inline int tile_ty(int B) { return B >= kTileInst ? 8 : 16; }
 // neighbouring rays, which on rays along x lie one pixel row apart; the swap puts them in different
 // parts of a bank line, as pixels one column apart are.
 __host__ __device__ inline int tile_slot(int q, int TX) { return q ^ ((q / TX) & 1); }
+// The layouts are an option: where device memory is short, or positions would not fit in 32 bits, the builders
+// return SGKS_OK with ntiles = 0 and leave nothing in allocs.  They run after everything that a handle cannot do
+// without.  tile_memory adds an array to allocs (the partial sums); both it and tile_room free all of allocs and
+// return false when memory is short, that is, when less than kTileRoom is left for graphs and modules
+// loaded later.
+constexpr size_t kTileRoom = (size_t)128 << 20;
+bool tile_room(std::vector<void*>& allocs);
+bool tile_memory(std::vector<void*>& allocs, void** p, size_t bytes);
+void drop_tile_memory(std::vector<void*>& allocs);
 int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t m, int64_t n, int64_t nnz, int nx, int ny,
                 int nt, int TX, int TY, TiledA& T, std::vector<void*>& allocs, cudaStream_t st, std::string* why);
 int build_tiles_t(const int32_t* trp, const int32_t* tci, const float* tval, int64_t m, int64_t n, int64_t nnz, int nx,
