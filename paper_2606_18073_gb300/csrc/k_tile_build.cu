@@ -1,6 +1,8 @@
 // Builds the tiled layouts of k_tiles.cu from a CSR operator, on the device.
 //
-// Both sides start from one bit per (tile, row of A): set when the row has an entry in the tile.  The
+// Both sides start from one bit per (tile, row of A): set when the row has an entry in the tile.  A tile has
+// bits for the range of rows that reach its frame (frames of a block-diagonal operator share no rows: bits for
+// all of them would grow with the square of the number of frames).  The
 // running bit count of a tile numbers its rows in ascending order ("local index").  Forward: the
 // (row, tile) segments are counted, sorted by length within the tile (stable), cut into groups of four
 // and filled by one warp per row, which walks the row's entries in order.  Transposed: the rows of a
@@ -18,9 +20,31 @@ namespace sgks {
 
 namespace {
 
+// Bits of the tiles of one frame: nw words a tile, tile by tile from word `base`, for the rows from 32 w0 on.
+struct FrameBits {
+    int64_t base;
+    int32_t w0, nw;
+};
+
 struct Geo {
-    int nx, ny, TX, TY, ntx, nty, ntiles;
-    int64_t n, m, words;   // words of a tile's bit row
+    int nx, ny, TX, TY, ntx, nty, ntiles, nt;
+    int64_t n, m;
+    const FrameBits* fb;   // [nt]
+    int64_t words;         // of all tiles
+    // first word of a tile; its first row (a multiple of 32) and its number of words
+    __device__ __forceinline__ size_t bits_of(int tile, int64_t* row0, int* nw) const {
+        const int tpf = ntx * nty, f = tile / tpf;
+        const FrameBits b = fb[f];
+        *row0 = (int64_t)b.w0 * 32;
+        *nw = b.nw;
+        return (size_t)b.base + (size_t)(tile - f * tpf) * b.nw;
+    }
+    __device__ __forceinline__ size_t word(int tile, int64_t row) const {
+        int64_t row0;
+        int nw;
+        const size_t w = bits_of(tile, &row0, &nw);
+        return w + (size_t)((row - row0) >> 5);
+    }
     __device__ __forceinline__ void locate(int64_t col, int* tile, int* loc) const {
         const int64_t fr = (int64_t)nx * ny, f = qdiv(col, fr), r = col - f * fr;
         const int iy = (int)qdiv(r, nx), ix = (int)(r - (int64_t)iy * nx);
@@ -30,9 +54,27 @@ struct Geo {
 };
 
 __device__ __forceinline__ void mark(uint32_t* bits, const Geo& g, int tile, int64_t row) {
-    uint32_t* w = bits + (size_t)tile * g.words + (row >> 5);
+    uint32_t* w = bits + g.word(tile, row);
     const uint32_t b = 1u << (row & 31);
     if (!(*(volatile uint32_t*)w & b)) atomicOr(w, b);
+}
+
+// Rows of A with an entry in frame f: lo[f] .. hi[f] (0x7f7f7f7f .. -1 without one), from the rows of A (by_row,
+// a warp per row) or from those of A^T (a warp per pixel).  Indices out of range are skipped.
+__global__ void k_frame_rows(Geo g, bool by_row, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, int64_t nnz,
+                             int32_t* lo, int32_t* hi) {
+    const int64_t GW = (int64_t)gridDim.x * kWarps, fr = (int64_t)g.nx * g.ny, rows = by_row ? g.m : g.n;
+    for (int64_t r = (int64_t)blockIdx.x * kWarps + warp_id(); r < rows; r += GW) {
+        const int32_t a = rp[r], z = rp[r + 1];
+        if (a < 0 || z < a || z > nnz) continue;
+        for (int32_t k = a + lane_id(); k < z; k += 32) {
+            const int32_t c = ci[k];
+            if (c < 0 || c >= (by_row ? g.n : g.m)) continue;
+            const int f = (int)qdiv(by_row ? c : r, fr), row = by_row ? (int)r : c;
+            if (row < *(volatile int32_t*)(lo + f)) atomicMin(lo + f, row);
+            if (row > *(volatile int32_t*)(hi + f)) atomicMax(hi + f, row);
+        }
+    }
 }
 
 // rows of A: a warp per row.  Column indices and row pointers out of range set err and are skipped.
@@ -82,12 +124,15 @@ __global__ void k_tile_mark_cols(Geo g, const int32_t* __restrict__ trp, const i
 __global__ void __launch_bounds__(kThreads) k_tile_count(Geo g, const uint32_t* __restrict__ bits, int32_t* before,
                                                          int32_t* cnt, int32_t* rows) {
     __shared__ int32_t part[kWarps];
-    const uint32_t* b = bits + (size_t)blockIdx.x * g.words;
-    int32_t* o = before + (size_t)blockIdx.x * g.words;
+    int64_t row0;
+    int nw;
+    const size_t first = g.bits_of(blockIdx.x, &row0, &nw);
+    const uint32_t* b = bits + first;
+    int32_t* o = before + first;
     int32_t base = 0;
-    for (int64_t w0 = 0; w0 < g.words; w0 += kThreads) {
-        const int64_t w = w0 + threadIdx.x;
-        const uint32_t v = w < g.words ? b[w] : 0u;
+    for (int w0 = 0; w0 < nw; w0 += kThreads) {
+        const int w = w0 + (int)threadIdx.x;
+        const uint32_t v = w < nw ? b[w] : 0u;
         int32_t inc = __popc(v);
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -102,9 +147,9 @@ __global__ void __launch_bounds__(kThreads) k_tile_count(Geo g, const uint32_t* 
             if (i < warp_id()) pre += part[i];
             tot += part[i];
         }
-        if (w < g.words) o[w] = base + pre + inc - __popc(v);
+        if (w < nw) o[w] = base + pre + inc - __popc(v);
         if (rows)
-            for (uint32_t x = v; x; x &= x - 1) atomicAdd(rows + w * 32 + (__ffs(x) - 1), 1);
+            for (uint32_t x = v; x; x &= x - 1) atomicAdd(rows + row0 + w * 32 + (__ffs(x) - 1), 1);
         base += tot;
         __syncthreads();
     }
@@ -113,7 +158,7 @@ __global__ void __launch_bounds__(kThreads) k_tile_count(Geo g, const uint32_t* 
 
 __device__ __forceinline__ int32_t local_index(const Geo& g, const uint32_t* __restrict__ bits,
                                                const int32_t* __restrict__ before, int tile, int64_t row) {
-    const size_t w = (size_t)tile * g.words + (row >> 5);
+    const size_t w = g.word(tile, row);
     return before[w] + __popc(bits[w] & ((1u << (row & 31)) - 1u));
 }
 
@@ -219,11 +264,14 @@ __global__ void k_seg_fill(Geo g, const int32_t* __restrict__ rp, const int32_t*
 // the rows of each tile in ascending order
 __global__ void k_tile_rays(Geo g, const uint32_t* __restrict__ bits, const int32_t* __restrict__ before,
                             const int32_t* __restrict__ tile_ray, int32_t* ray) {
-    const uint32_t* b = bits + (size_t)blockIdx.x * g.words;
-    const int32_t* o = before + (size_t)blockIdx.x * g.words;
-    for (int64_t w = threadIdx.x; w < g.words; w += blockDim.x) {
+    int64_t row0;
+    int nw;
+    const size_t first = g.bits_of(blockIdx.x, &row0, &nw);
+    const uint32_t* b = bits + first;
+    const int32_t* o = before + first;
+    for (int w = threadIdx.x; w < nw; w += blockDim.x) {
         int32_t p = tile_ray[blockIdx.x] + o[w];
-        for (uint32_t x = b[w]; x; x &= x - 1) ray[p++] = (int32_t)(w * 32 + (__ffs(x) - 1));
+        for (uint32_t x = b[w]; x; x &= x - 1) ray[p++] = (int32_t)(row0 + w * 32 + (__ffs(x) - 1));
     }
 }
 
@@ -332,10 +380,36 @@ std::vector<int32_t> heavy_first(const std::vector<int32_t>& off, const std::vec
 
 bool geometry(int64_t m, int64_t n, int nx, int ny, int nt, int TX, int TY, Geo* g) {
     if ((int64_t)nx * ny * nt != n) return false;
-    *g = Geo{nx, ny, TX, TY, (nx + TX - 1) / TX, (ny + TY - 1) / TY, 0, n, m, (m + 31) / 32};
+    *g = Geo{nx, ny, TX, TY, (nx + TX - 1) / TX, (ny + TY - 1) / TY, 0, nt, n, m, nullptr, 0};
     const int64_t tiles = (int64_t)g->ntx * g->nty * nt;
     g->ntiles = (int)tiles;
     return tiles < ((int64_t)1 << 31);
+}
+
+// g.fb and g.words; one frame takes bits for all rows without looking at the entries
+void frame_bits(Build& b, Geo& g, bool by_row, const int32_t* rp, const int32_t* ci, int64_t nnz) {
+    std::vector<int32_t> lo((size_t)g.nt, 0), hi((size_t)g.nt, (int32_t)(g.m - 1));
+    if (g.nt > 1) {
+        int32_t *dlo = b.temp<int32_t>(g.nt), *dhi = b.temp<int32_t>(g.nt);
+        if (b.e == cudaSuccess) b.e = cudaMemsetAsync(dlo, 0x7f, 4 * (size_t)g.nt, b.st);
+        if (b.e == cudaSuccess) b.e = cudaMemsetAsync(dhi, 0xff, 4 * (size_t)g.nt, b.st);
+        if (b.e != cudaSuccess) return;
+        const int64_t rows = by_row ? g.m : g.n;
+        k_frame_rows<<<grid_for((rows + kWarps - 1) / kWarps), kThreads, 0, b.st>>>(g, by_row, rp, ci, nnz, dlo, dhi);
+        b.ran();
+        lo = b.down(dlo, g.nt);
+        hi = b.down(dhi, g.nt);
+    }
+    std::vector<FrameBits> h((size_t)g.nt);
+    for (int f = 0; f < g.nt; ++f) {
+        const int32_t w0 = hi[f] < 0 ? 0 : lo[f] / 32, nw = hi[f] < 0 ? 0 : hi[f] / 32 - w0 + 1;
+        h[f] = FrameBits{g.words, w0, nw};
+        g.words += (int64_t)nw * g.ntx * g.nty;
+    }
+    FrameBits* d = b.temp<FrameBits>(g.nt);
+    if (b.e == cudaSuccess) b.e = cudaMemcpyAsync(d, h.data(), sizeof(FrameBits) * h.size(), cudaMemcpyHostToDevice, b.st);
+    if (b.e == cudaSuccess) b.e = cudaStreamSynchronize(b.st);   // the host vector dies
+    g.fb = d;
 }
 
 // Without the memory for a layout the row kernels remain, which need none of it: no error.
@@ -383,14 +457,15 @@ int build_tiles(const int32_t* rp, const int32_t* ci, const float* val, int64_t 
     Geo g;
     if (TX % 2 != 0 || nnz >= ((int64_t)1 << 31) || !geometry(m, n, nx, ny, nt, TX, TY, &g))
         return refused(why, "geometry does not match the unknowns");
-    const size_t nw = (size_t)g.ntiles * g.words;
-    if (nw > kMaxWords) return SGKS_OK;
     Build b(st);
+    frame_bits(b, g, true, rp, ci, nnz);
+    const size_t nw = (size_t)g.words, row_words = (size_t)(m + 31) / 32 * 32;
+    if (nw > kMaxWords) return SGKS_OK;
     uint32_t* bits = b.temp<uint32_t>(nw);
-    int32_t *before = b.temp<int32_t>(nw), *cnt = b.temp<int32_t>(g.ntiles), *rows = b.temp<int32_t>(g.words * 32);
+    int32_t *before = b.temp<int32_t>(nw), *cnt = b.temp<int32_t>(g.ntiles), *rows = b.temp<int32_t>(row_words);
     int32_t* err = b.temp<int32_t>(1);
     b.zero(bits, nw * 4);
-    b.zero(rows, g.words * 32 * 4);
+    b.zero(rows, row_words * 4);
     b.zero(err, 4);
     if (b.e != cudaSuccess) return failed(b, why);
     const unsigned gr = grid_for((m + kWarps - 1) / kWarps);
@@ -438,9 +513,10 @@ int build_tiles_t(const int32_t* trp, const int32_t* tci, const float* tval, int
     Geo g;
     if (nnz >= ((int64_t)1 << 31) || !geometry(m, n, nx, ny, nt, TX, TY, &g))
         return refused(why, "geometry does not match the unknowns");
-    const size_t nw = (size_t)g.ntiles * g.words;
-    if (nw > kMaxWords) return SGKS_OK;
     Build b(st);
+    frame_bits(b, g, false, trp, tci, nnz);
+    const size_t nw = (size_t)g.words;
+    if (nw > kMaxWords) return SGKS_OK;
     uint32_t* bits = b.temp<uint32_t>(nw);
     int32_t *before = b.temp<int32_t>(nw), *cnt = b.temp<int32_t>(g.ntiles), *err = b.temp<int32_t>(1);
     b.zero(bits, nw * 4);
