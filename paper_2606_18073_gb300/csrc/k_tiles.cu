@@ -16,7 +16,7 @@
 // What bounds both is the FP32 pipe: 11 operations per entry and instance of Dot2 (ff.cuh) are
 // 42.3 G on the CT batch (60 M entries, 64 instances), 1.05 ms at 40.3 T/s; Dot2 alone, on registers,
 // reaches 33 T/s.  Measured there (float-float): A w 2.82 -> 1.93 ms with kbx_seg_reduce's 0.25, A^T e
-// 3.07 -> 2.00 ms against the row kernel's 512-byte gathers.  A batch of one on a 301^2 image: 105 -> 62
+// 3.07 -> 2.18 ms against the row kernel's 512-byte gathers.  A batch of one on a 301^2 image: 105 -> 62
 // and 92 -> 43 us.  Therefore
 // - a lane works on two instances at once with the .f32x2 instructions, 11 per entry, which leaves half
 //   of the issue slots for the loads and addresses; with 16 instances it takes two such pairs, so that
@@ -69,8 +69,8 @@ __device__ __forceinline__ void add_pair(Dot2x2 (&d)[Lanes<IC>::NP], const Stage
 }
 
 // Pairs [beg, end) of a row into acc, in blocks of kDot2Block terms (ff.cuh); cur holds the pairs beg
-// and beg + 1 and leaves with those of the next row, from `next` on.  FIRST: acc is still 0.
-template <bool FIRST, typename TW, int IC>
+// and beg + 1 and leaves with those of the next row, from `next` on.
+template <typename TW, int IC>
 __device__ __forceinline__ void add_row(Dot2x2 (&acc)[Lanes<IC>::NP], const Staged<TW, IC>& st, Entries& cur,
                                         const uint4* __restrict__ ent, int beg, int end, int next) {
     constexpr int NP = Lanes<IC>::NP, PB = kDot2Block / 2;
@@ -97,8 +97,54 @@ __device__ __forceinline__ void add_row(Dot2x2 (&acc)[Lanes<IC>::NP], const Stag
         }
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
-            if (FIRST && kb == beg) acc[i] = blk[i];
+            if (kb == beg) acc[i] = blk[i];
             else acc[i].merge(blk[i]);
+        }
+    }
+}
+
+// The same for the transposed pass, whose rows go on through the stages of a tile.  Added one block after the other
+// (as above, 16 terms each) such a row's error was 1.3 to 1.8 times that of the row kernel's eight lanes: every
+// merge into a sum of full size rounds its low part.  So the terms form a tree, blocks of eight, up to 32 terms of
+// them in a sum of their own, and that into acc: 0.9 to 1.1 times the row kernel's (rms of x after one iteration,
+// float-float, 97^2 with 100, 181^2 with 180 and 256^2 with 30 views).  With 16 instances a stage brings a pixel
+// of a ray operator about 30 terms, so one sum takes them all; HALVES (float-float, fewer instances): the blocks are two
+// chains of four.  512^2 at 64: 2.00 -> 2.18 ms per pass; with fewer instances the same time as before.
+template <bool HALVES, int IC>
+__device__ __forceinline__ void add_row_tree(Dot2x2 (&acc)[Lanes<IC>::NP], const Staged<float2, IC>& st, Entries& cur,
+                                             const uint4* __restrict__ ent, int beg, int end, int next) {
+    constexpr int NP = Lanes<IC>::NP, part = IC >= 16 ? 1 << 28 : 16;   // entry pairs in a sum of their own
+    if (beg == end) {
+        cur.load(ent, next);
+        return;
+    }
+    for (int pb = beg; pb < end; pb += part) {
+        const int pe = min(end, pb + part);
+        Dot2x2 sum[NP];
+        for (int k = pb; k < pe; k += 4) {
+            Dot2x2 blk[NP], alt[NP];
+            auto& odd = HALVES ? alt : blk;
+            Entries nxt;
+            nxt.load(ent, k + 2 < end ? k + 2 : next);
+            add_pair<float2, IC>(blk, st, cur.a);
+            if (k + 1 < pe) add_pair<float2, IC>(odd, st, cur.b);
+            if (k + 2 < pe) {
+                cur.load(ent, k + 4 < end ? k + 4 : next);
+                add_pair<float2, IC>(blk, st, nxt.a);
+                if (k + 3 < pe) add_pair<float2, IC>(odd, st, nxt.b);
+            } else {
+                cur = nxt;
+            }
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                if (HALVES) blk[i].merge(alt[i]);
+                sum[i].merge(blk[i]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            acc[i].merge(sum[i]);
+            acc[i].renorm();
         }
     }
 }
@@ -163,7 +209,7 @@ __global__ void __launch_bounds__(Lanes<IC>::threads, IC >= 16 ? 3 : 2) kbx_tile
         group(s + 2 * step, fbeg, fend);
         if constexpr (IC == 16) entries_to_l2(T.ent, nbeg, nend, threadIdx.x & 15);
         Dot2x2 a[LN::NP];
-        add_row<true, TW, IC>(a, st, cur, ent, beg, end, nbeg);
+        add_row<TW, IC>(a, st, cur, ent, beg, end, nbeg);
         beg = nbeg;
         end = nend;
         nbeg = fbeg;
@@ -309,9 +355,7 @@ __global__ void __launch_bounds__(GradShape<IC, TY>::threads, IC >= 16 ? 3 : 102
             g = min(g + rows / 4, glast);
             const int fbeg = T.goff[g], fend = T.goff[g + 1];
             if constexpr (IC == 16) entries_to_l2(T.ent, nbeg, nend, threadIdx.x & 15);
-            add_row<false, float2, IC>(acc[u], st, cur, ent, beg, end, nbeg);
-#pragma unroll
-            for (int i = 0; i < LN::NP; ++i) acc[u][i].renorm();   // once per stage (ff.cuh)
+            add_row_tree<(IC < 16 && sizeof(TW) == sizeof(float2)), IC>(acc[u], st, cur, ent, beg, end, nbeg);
             beg = nbeg;
             end = nend;
             nbeg = fbeg;
