@@ -61,6 +61,27 @@ __global__ void kd_axpby(T* out, const T* x, double alpha, const T* y, double be
         out[i] = (T)(alpha * (double)x[i] + (y ? beta * (double)y[i] : 0.0));
 }
 
+// *bits = the largest |x[i]| as a bit pattern (which orders like the values; infinities and NaN on top)
+__global__ void __launch_bounds__(kThreads) kd_absmax(const double* __restrict__ x, int64_t n, unsigned long long* bits) {
+    unsigned long long m = 0;
+    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads)
+        m = max(m, (unsigned long long)__double_as_longlong(x[i]) & 0x7fffffffffffffffull);
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane_id() == 0 && m) atomicMax(bits, m);
+}
+
+// x *= 2^(-e) (back: 2^e) with e the exponent of *bits, within +-1000; nothing for 0, infinities and NaN.  acc: one
+// more value, or null.
+__global__ void __launch_bounds__(kThreads) kd_scale_pow2(double* x, int64_t n, const unsigned long long* bits, bool back,
+                                                          double* acc) {
+    const int field = (int)(*bits >> 52);
+    if (*bits == 0 || field == 0x7ff) return;
+    const int e = max(-1000, min(1000, field - 1023));
+    const double f = __hiloint2double((1023 + (back ? e : -e)) << 20, 0);
+    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) x[i] *= f;
+    if (acc && blockIdx.x == 0 && threadIdx.x == 0) *acc *= f;
+}
+
 // FP64 s-vectors: out = alpha x + beta y
 __global__ void kd_axpby_d(double* out, const double* x, double alpha, const double* y, double beta, int n) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
@@ -208,6 +229,19 @@ cudaError_t launchd_rank2(T* Wb, int64_t n, int d, const T* a, const double* p, 
 template <typename T>
 cudaError_t launchd_axpby(T* out, const T* x, double alpha, const T* y, double beta, int64_t n, cudaStream_t st) {
     kd_axpby<T><<<agrid(n), kThreads, 0, st>>>(out, x, alpha, y, beta, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launchd_scale_down(double* x, int64_t n, unsigned long long* bits, cudaStream_t st) {
+    const cudaError_t e = cudaMemsetAsync(bits, 0, sizeof(*bits), st);
+    if (e != cudaSuccess) return e;
+    kd_absmax<<<agrid(n), kThreads, 0, st>>>(x, n, bits);
+    kd_scale_pow2<<<agrid(n), kThreads, 0, st>>>(x, n, bits, false, nullptr);
+    return cudaGetLastError();
+}
+
+cudaError_t launchd_scale_back(double* x, int64_t n, const unsigned long long* bits, double* acc, cudaStream_t st) {
+    kd_scale_pow2<<<agrid(n), kThreads, 0, st>>>(x, n, bits, true, acc);
     return cudaGetLastError();
 }
 

@@ -11,7 +11,8 @@
 // - a conversion from FP32 costs as much as a multiply-add, so a value's bits are only moved into place: as
 //   a double they are a 2^-896 exactly (FP32 subnormals included).  Staged values are multiplied by 2^448
 //   and sums by 2^448 once each, which leaves products between 2^-574 and 2^576 exact; outside of
-//   that the solver's squared norms have under- or overflowed before.  An operator with infinite or NaN values
+//   that the solver's squared norms have under- or overflowed before, and the reverse sweep, which takes no such
+//   norms, scales its cotangent and keeps its Krylov vectors on the row kernels (sgks_api.cu).  An operator with infinite or NaN values
 //   keeps the row kernels (build_tiles64), and so does one with fewer than 2^20 entries;
 // - with several instances a lane takes up to four of them, for one entry load and one set of bit moves.
 #include <algorithm>

@@ -294,6 +294,7 @@ struct Engine : EngineBase {
         T *Ww = nullptr, *HWw = nullptr, *xp = nullptr, *rho = nullptr, *a1 = nullptr, *a2 = nullptr;
         T *xin = nullptr, *bout = nullptr;   // the caller's xbar and the result bbar, copied in and out
         int* err = nullptr;
+        unsigned long long* amax = nullptr;  // scale of the cotangent (tiled passes)
     } bw;
     // The sweep for one (K, lambda) as a CUDA graph: the first call for a key runs the launches
     // eagerly, the second captures them, later calls replay the graph.
@@ -340,7 +341,7 @@ struct Engine : EngineBase {
         A1(&bw.P, n); A1(&bw.Q, n); A1(&bw.tm, m); A1(&bw.tp, p); A1(&bw.Kv, ell * n); A1(&bw.Kb, ell * n);
         A1(&bw.uy, s); A1(&bw.uz, s); A1(&bw.vy, s); A1(&bw.vz, s); A1(&bw.cb, s); A1(&bw.st, s);
         A1(&bw.ybar, dm); A1(&bw.z, dm); A1(&bw.part, (size_t)nbS * dm); A1(&bw.acc, 2);
-        A1(&bw.R0, ell * ell); A1(&bw.Ri, ell * ell); A1(&bw.err, 1); A1(&bw.xin, n); A1(&bw.bout, m);
+        A1(&bw.R0, ell * ell); A1(&bw.Ri, ell * ell); A1(&bw.err, 1); A1(&bw.amax, 1); A1(&bw.xin, n); A1(&bw.bout, m);
         if (n_refine > 0) {
             A1(&bw.w, dm); A1(&bw.dl, dm); A1(&bw.td, dm);
             A1(&bw.Ww, n); A1(&bw.HWw, n); A1(&bw.xp, n); A1(&bw.rho, n); A1(&bw.a1, n); A1(&bw.a2, n);
@@ -364,6 +365,32 @@ struct Engine : EngineBase {
     cudaError_t bw_apply(int which, const T* in, T* out) {
         g_launches.fetch_add(1);
         return op_apply(which, in, out);
+    }
+
+    // Range of the tiled passes (k_tiles64.cu) in the sweep: its vectors are linear in the cotangent, whose scale is
+    // the caller's, so that is brought to 1 by a power of two (bw_scale; bw_unscale takes it off the results,
+    // all roundings are the same).  The Krylov vectors at its end are not normalised, up to ||A||^5 ||b||: those
+    // passes stay on the row kernels (bw_apply_full).
+    bool tiled() const { return Ta.ntiles != 0; }
+    cudaError_t bw_scale() {
+        if constexpr (std::is_same<T, double>::value) {
+            if (!tiled()) return cudaSuccess;
+            g_launches.fetch_add(2);
+            return launchd_scale_down(bw.xb, D.n, bw.amax, st);
+        }
+        return cudaSuccess;
+    }
+    cudaError_t bw_unscale() {
+        if constexpr (std::is_same<T, double>::value) {
+            if (!tiled()) return cudaSuccess;
+            g_launches.fetch_add(1);
+            return launchd_scale_back(bw.bout, D.m, bw.amax, bw.acc, st);
+        }
+        return cudaSuccess;
+    }
+    cudaError_t bw_apply_full(int which, const T* in, T* out) {
+        g_launches.fetch_add(1);
+        return launch_apply<T, V>(D, A, L, which, in, out, st);
     }
 
     cudaError_t bw_sketch_adj(bool isA, const double* u, T* out) {
@@ -494,6 +521,7 @@ struct Engine : EngineBase {
         if (e == cudaSuccess) e = cudaMemsetAsync(bw.err, 0, sizeof(int), st);
         if (e == cudaSuccess) e = cudaMemsetAsync(bbar, 0, sizeof(T) * D.m, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(bw.xb, bw.xin, sizeof(T) * n, cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess) e = bw_scale();
         auto L1 = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
         const int NS = n_refine + 1;
         auto yrow = [&](int j, int r) { return yhist + ((size_t)j * NS + r) * D.dmax; };
@@ -552,10 +580,10 @@ struct Engine : EngineBase {
         for (int i = 0; i < ell && e == cudaSuccess; ++i) {
             T* Ki = bw.Kv + (size_t)i * n;
             if (i == 0) {
-                L1(bw_apply(SGKS_APPLY_AT, b_own, Ki));
+                L1(bw_apply_full(SGKS_APPLY_AT, b_own, Ki));
             } else {
-                L1(bw_apply(SGKS_APPLY_A, bw.Kv + (size_t)(i - 1) * n, bw.tm));
-                L1(bw_apply(SGKS_APPLY_AT, bw.tm, Ki));
+                L1(bw_apply_full(SGKS_APPLY_A, bw.Kv + (size_t)(i - 1) * n, bw.tm));
+                L1(bw_apply_full(SGKS_APPLY_AT, bw.tm, Ki));
             }
             L1(bw_dots(W, ell, Ki, bw.R0 + (size_t)i * ell));
         }
@@ -565,16 +593,17 @@ struct Engine : EngineBase {
         // vbar = sum_i (A^T A)^i Kbar_i by Horner, into t1
         L1(cudaMemcpyAsync(bw.t1, bw.Kb + (size_t)(ell - 1) * n, sizeof(T) * n, cudaMemcpyDeviceToDevice, st));
         for (int i = ell - 2; i >= 0 && e == cudaSuccess; --i) {
-            L1(bw_apply(SGKS_APPLY_A, bw.t1, bw.tm));
-            L1(bw_apply(SGKS_APPLY_AT, bw.tm, bw.t2));
+            L1(bw_apply_full(SGKS_APPLY_A, bw.t1, bw.tm));
+            L1(bw_apply_full(SGKS_APPLY_AT, bw.tm, bw.t2));
             L1(launchd_axpby<T>(bw.t1, bw.Kb + (size_t)i * n, 1.0, bw.t2, 1.0, n, st));
             g_launches.fetch_add(1);
         }
-        L1(bw_apply(SGKS_APPLY_A, bw.t1, bw.tm));
+        L1(bw_apply_full(SGKS_APPLY_A, bw.t1, bw.tm));
         L1(launchd_axpby<T>(bbar, bbar, 1.0, bw.tm, 1.0, D.m, st));
         L1(bw_sketch_adj(true, bw.cb, bw.tm));
         L1(launchd_axpby<T>(bbar, bbar, 1.0, bw.tm, 1.0, D.m, st));
         g_launches.fetch_add(2);
+        L1(bw_unscale());
         return e;
     }
 

@@ -1156,6 +1156,10 @@ cudaError_t launchd_rank2(T* Wb, int64_t n, int d, const T* a, const double* p, 
                           cudaStream_t st);
 template <typename T>
 cudaError_t launchd_axpby(T* out, const T* x, double alpha, const T* y, double beta, int64_t n, cudaStream_t st);
+// x scaled by the power of two that brings its largest element to [1, 2), kept in *bits; and the scale taken off
+// another vector and off *acc again
+cudaError_t launchd_scale_down(double* x, int64_t n, unsigned long long* bits, cudaStream_t st);
+cudaError_t launchd_scale_back(double* x, int64_t n, const unsigned long long* bits, double* acc, cudaStream_t st);
 cudaError_t launchd_axpby_d(double* out, const double* x, double alpha, const double* y, double beta, int n,
                             cudaStream_t st);
 cudaError_t launchd_dot_acc(const double* a, const double* b, int len, double sign, double* acc, cudaStream_t st);
