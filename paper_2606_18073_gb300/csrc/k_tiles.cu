@@ -407,7 +407,7 @@ static cudaError_t tile_apply_ic(const BDims& D, const TiledA& T, const BBulkX<T
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     constexpr int NB = IC == 1 ? 1 : 2;
-    const int lanes = seg_lanes(D.B / NB, D.alone);
+    const int lanes = seg_lanes(D.B / NB);
     const int64_t rb = (D.m * (D.B / NB) * lanes + kThreads - 1) / kThreads;
     kbx_seg_reduce<TW, NB><<<(int)std::max<int64_t>(1, std::min<int64_t>(rb, 8 * 152)), kThreads, 0, st>>>(D, T, X, S, part, lanes);
     return cudaGetLastError();

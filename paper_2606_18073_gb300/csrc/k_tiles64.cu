@@ -235,7 +235,7 @@ cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileV
         default: e = apply64_ic<16>(T, W, part, st); break;
     }
     if (e != cudaSuccess) return e;
-    const int lanes = seg_lanes(W.B, alone);
+    const int lanes = seg_lanes(W.B);
     const int nbu = (int)std::max<int64_t>(1, std::min<int64_t>((m * W.B * lanes + kThreads - 1) / kThreads, 8 * 152));
     const int nbl = lw ? (int)std::max<int64_t>(1, std::min<int64_t>((L.p + kThreads - 1) / kThreads, 8 * 152)) : 0;
     return launch_pdl(kd_seg_reduce, nbu + nbl, kThreads, 0, st, T, U, m, part, lanes, nbu, L, W, lw);

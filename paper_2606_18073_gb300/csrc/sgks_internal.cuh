@@ -978,10 +978,11 @@ struct PtrPack {
 
 // Lanes that share a ray of n instance lanes in the sums over segments, within a warp: a ray of a CT image crosses
 // some 20 to 60 tiles, and eight lanes leave each one round or two of loads.  512^2, FP64, one vector: 45 -> 20 us;
-// a batch of one, float-float, 301^2: 17 -> 11 us.  A batch of several groups runs them next to each other and
-// fills the chip without, where merging costs more than waiting (7.61 against 7.72 ms per solve of 11 slices of
-// 243^2): one lane there.
-inline int seg_lanes(int n, bool alone) { return !alone || n >= 32 ? 1 : std::min(8, 32 / n); }
+// a batch of one, float-float, 301^2: 17 -> 11 us.  The lanes set the order of a ray's sum, so they follow from n
+// alone: a batch of several groups, which run next to each other and fill the chip without, would be a little faster
+// with one lane (7.61 against 7.72 ms per solve of 11 slices of 243^2), but an instance's result would
+// then depend on what else is in the batch.
+inline int seg_lanes(int n) { return n >= 32 ? 1 : std::min(8, 32 / n); }
 
 template <typename T, typename V>
 cudaError_t launchb_apply_column(const BDims& D, const DevA<T, V>& A, const DevL& L, const BBulk<T>& X,
