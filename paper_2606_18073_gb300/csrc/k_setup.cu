@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kThreads) k_dots_plain(const T* __restrict__ V
                 err += (s - (t - bb)) + (red[q] - bb);
                 s = t;
             }
-            part[(size_t)blockIdx.x * k + c] = s + err;
+            part[(size_t)blockIdx.x * k + c] = isfinite(s) ? s + err : s;   // infinite: err is NaN
         }
         __syncthreads();
     }
