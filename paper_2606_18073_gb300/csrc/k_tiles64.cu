@@ -29,6 +29,16 @@ __device__ __forceinline__ double tiny_bits(uint32_t f) {   // the FP32 value wi
     return __hiloint2double((int)(((f >> 3) & 0x0fffffffu) | (f & 0x80000000u)), (int)(f << 29));
 }
 
+// v 2^448 for the shared memory, for a vector that comes from the caller (b at the setup): what would overflow, finite
+// values from 2^575 on, stays finite at 2^1023.  The squared norm is infinite in any case, and the solver then
+// ends as it does with the row kernels, in a breakdown (infinite elements would make its first column NaN).
+// Elsewhere such values end a solve either way; all staged values that way cost 1.6 % of a solve (16 instances, 256^2).
+__device__ __forceinline__ double to_stage(double v) {
+    const int hi = __double2hiint(v), field = (hi >> 20) & 0x7ff;
+    const double r = v * kHalfScale;
+    return field >= 1023 + 575 && field != 0x7ff ? __hiloint2double((hi & 0x80000000) | 0x7fe00000, 0) : r;
+}
+
 template <int IC>
 struct Lanes64 {
     static constexpr int VV = IC >= 4 ? 4 : IC, G = IC / VV, rows = kThreads / G;
@@ -179,7 +189,10 @@ __global__ void __launch_bounds__(kThreads, 3) kd_tile_gradient(TiledT T, TileVe
             const double* src = E.p + (size_t)(q < nr ? T.ray[r0 + q] : 0) * B + b0;
             double* dst = es + (q < nr ? q : T.stage) * IC + lane0;   // slot T.stage holds 0
 #pragma unroll
-            for (int v = 0; v < LN::VV; ++v) dst[v] = q < nr ? __ldcg(src + v) * kHalfScale : 0.0;
+            for (int v = 0; v < LN::VV; ++v) {
+                const double ev = q < nr ? __ldcg(src + v) : 0.0;
+                dst[v] = sc ? ev * kHalfScale : to_stage(ev);
+            }
         }
         __syncthreads();
 #pragma unroll
