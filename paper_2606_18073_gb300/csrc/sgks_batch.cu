@@ -12,6 +12,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <functional>
 #include <map>
 #include <mutex>
@@ -58,20 +59,12 @@ struct GroupBase {
     std::string tuned;   // the configuration the tuner chose (for sgks_batch_tuning)
 };
 
-// Autotuner cache: one entry per (operator shape, nonzeros, group size, precision).
-struct TuneKey {
-    int64_t m, n, p, nnz;
-    int B, elem, kind;
-    bool operator<(const TuneKey& o) const {
-        if (m != o.m) return m < o.m;
-        if (n != o.n) return n < o.n;
-        if (p != o.p) return p < o.p;
-        if (nnz != o.nnz) return nnz < o.nnz;
-        if (B != o.B) return B < o.B;
-        if (elem != o.elem) return elem < o.elem;
-        return kind < o.kind;
-    }
-};
+// Autotuner cache: one entry per (operator shape, nonzeros, image, group size, precision, and the width and height of
+// the tiles of A and of A^T, 0 for the row kernels: what there is to tune depends on them).
+using TuneKey = std::array<int64_t, 12>;
+TuneKey tune_key(const BDims& D, int64_t nnz, const DevL& L, int elem, int kind, const TiledA& Ta, const TiledT& Tt) {
+    return {D.m, D.n, D.p, nnz, L.nx, L.ny, L.nt, D.B, elem, kind, Ta.ntiles ? Ta.TX : 0, Tt.ntiles ? Tt.TY : 0};
+}
 struct TuneVal {
     int slice_kb, nl_a, nl_t, tile_ic;
 };
@@ -230,7 +223,7 @@ struct Group : GroupBase {
     // lanes per CSR row for A and A^T (1 .. 32).  The kernels only rewrite state that the next
     // iteration recomputes from the same inputs.  Results are cached per shape and group size.
     cudaError_t tune() override {
-        const TuneKey key{D.m, D.n, D.p, A.kind == SGKS_OP_CSR ? nnz : 0, D.B, (int)sizeof(T), A.kind};
+        const TuneKey key = tune_key(D, nnz, L, (int)sizeof(T), A.kind, Ta, Tt);
         {
             std::lock_guard<std::mutex> g(g_tune_mu);
             auto it = g_tune_cache.find(key);
@@ -458,7 +451,7 @@ struct GroupX : GroupBase {
 
     // The tuner of Group: bulk-copy slice of the combine, lanes per CSR row of A and A^T.
     cudaError_t tune() override {
-        const TuneKey key{D.m, D.n, D.p, A.kind == SGKS_OP_CSR ? nnz : 0, D.B, 100 + (int)sizeof(TW), A.kind};
+        const TuneKey key = tune_key(D, nnz, L, 100 + (int)sizeof(TW), A.kind, T, Tt);
         {
             std::lock_guard<std::mutex> g(g_tune_mu);
             auto it = g_tune_cache.find(key);
