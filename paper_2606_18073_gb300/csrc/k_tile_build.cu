@@ -576,6 +576,14 @@ int build_tiles64(const sgks_reg* reg, const int32_t* rp, const int32_t* ci, con
     if (reg->kind == SGKS_REG_FD1 || nnz < (1 << 20)) return SGKS_OK;
     const int nt = reg->kind == SGKS_REG_SPACETIME ? reg->nt : 1;
     if ((int64_t)reg->nx * reg->ny * nt != n) return SGKS_OK;
+    // A CTA of the transposed pass holds a tile, for eight instances at most, so a small image with many rays leaves
+    // most of the chip idle, where the row kernels fill it.  Solves of 12 iterations against the row kernels
+    // (CT, 90 and 300 views; CTAs): one vector 0.90 (16), 1.01 (25), 1.10-1.17 (49); groups of 2 to 8, also
+    // 8 + 2 + 1, 0.55-1.0 (49), 0.87-1.1 (64), 0.86-1.16 (81), 0.96-1.23 (100), 1.02-1.3 (144); of 16 and more, also
+    // 16 + 1, 0.88-1.1 (64), 0.95-1.2 (182), 0.98-1.27 (196), 1.1-1.36 (256).
+    const int64_t grad_ctas = (int64_t)((reg->nx + kTileTX - 1) / kTileTX) * ((reg->ny + tile_ty(B) - 1) / tile_ty(B)) * nt *
+                              std::max(1, B / 8);
+    if (grad_ctas < (B == 1 ? 24 : (B < kTileInst ? 128 : 224))) return SGKS_OK;
     {
         Build b(st);
         int32_t* bad = b.temp<int32_t>(1);

@@ -1086,8 +1086,9 @@ cudaError_t launch64_tile_apply(const TiledA& T, const TileVec64& W, const TileV
 // sc given: instances that have stopped are left out.
 cudaError_t launch64_tile_gradient(const TiledT& T, const TileVec64& E, const TileVec64& O, DevScalars* sc, const DevL& L,
                                    const double* x, const double* lam, double lam1, cudaStream_t st);
-// Both layouts for FP64 vectors where they pay: a CSR operator with finite FP32 values and 2^20 entries or more
-// on an image (the regularizer's), whose rows share tiles; else T.ntiles = Tt.ntiles = 0.  B: largest group.
+// Both layouts for FP64 vectors where they pay: a CSR operator with finite FP32 values and 2^20 entries or more (1.26
+// to 1.47 times the row kernels at 1.3 M entries; smaller ones were not measured) on an image (the regularizer's)
+// of enough tiles, whose rows share tiles; else T.ntiles = Tt.ntiles = 0.  B: largest group.
 int build_tiles64(const sgks_reg* reg, const int32_t* rp, const int32_t* ci, const float* val, const int32_t* trp,
                   const int32_t* tci, const float* tval, int64_t m, int64_t n, int64_t nnz, int B, TiledA& T, TiledT& Tt,
                   std::vector<void*>& allocs, cudaStream_t st, std::string* why);

@@ -20,13 +20,13 @@ def G():
 
 @pytest.mark.parametrize("scale", [1e160, 1e200, 1e300])
 def test_large_data(G, scale):
-    A = ct_op(150, np.arange(60) * 3.0, 213)
+    A = ct_op(192, np.arange(40) * 4.5, 275)
     assert A.val.size >= 1 << 20
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
     C = G.CSR(dev(A.row_ptr), dev(A.col), dev(A.val.astype(np.float32)), A.m, A.n).transposed()
     rng = np.random.default_rng(1)
     b, plain = dev(rng.uniform(0.5, 1.5, A.m)) * scale, dev(rng.uniform(0.5, 1.5, A.m))
-    reg = G.Reg("grad2d", 150, 150)
+    reg = G.Reg("grad2d", 192, 192)
     S = G.Solver(C, reg, b, 1.0, 60, 3, max_iters=4)
     assert S.status() == 1     # SGKS_BREAKDOWN
     S.close()

@@ -17,7 +17,7 @@ def G():
     return G
 
 
-@pytest.mark.parametrize("prec,count,N", [("ff", 16, 45), ("fp64", 4, 97)])
+@pytest.mark.parametrize("prec,count,N", [("ff", 16, 45), ("fp64", 4, 192)])
 @pytest.mark.parametrize("first", [True, False])
 def test_tiled_and_row_passes_are_tuned_apart(G, prec, count, N, first):
     A = ct_op(N, np.arange(100) * 1.8, int(1.43 * N) + int(first))   # a shape of its own per order
