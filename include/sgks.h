@@ -143,15 +143,23 @@ typedef struct sgks_options {
                              instances per CTA of the tiled forward pass, the default or half of it),
                              a candidate replacing the default only when at least 5% faster;
                              results are cached per shape for the process.  Without it the
-                             defaults are used (16 KB, 8, 8; 16 instances per tile CTA) and results are reproducible from run to run; the slice
-                             and the tile instances keep every sum's order, the lanes per CSR row
-                             change it (at the level of rounding).
-                             bit 4 (SGKS_FLAG_NO_TILES, batches only): the compensated forms
-                             (FP32, FF) compute A w of a CSR operator whose regularizer gives an
-                             image geometry (2D stencils, space-time) through pixel tiles: each
-                             tile of w is staged once in shared memory and the rays crossing it
-                             leave one partial sum per (ray, tile), summed per ray in entry
-                             order.  This flag keeps the CSR-row kernel instead.
+                             defaults are used (16 KB, 8, 8; 16 instances per tile CTA) and
+                             results are reproducible from run to run; the slice and the tile
+                             instances keep every sum's order, the lanes per CSR row change it (at
+                             the level of rounding).
+                             bit 4 (SGKS_FLAG_NO_TILES, batches only): batches of the compensated
+                             forms (FP32, FF), and of FP64 from 2^20 entries and a few dozen tiles
+                             on (FP32 values, all finite), apply a CSR operator whose regularizer
+                             gives an image geometry (2D stencils, space-time) through pixel tiles.
+                             A w: each tile of w is staged once in shared memory and the rays
+                             crossing it leave one partial sum per (ray, tile), which up to
+                             eight lanes add up ray by ray (a fixed order that follows from the
+                             group's size).  A^T e: the rays crossing a tile are staged and every
+                             pixel adds up its entries.  The layouts take about 8 bytes per
+                             entry each; where device memory has no room for them the CSR-row
+                             kernels are used, and this flag keeps those always.  Single FP64
+                             handles use the tiles by the same rules, without a flag; results
+                             differ from the row kernels' at the level of rounding.
                              bit 5 (SGKS_FLAG_BW_HOST, with SGKS_FLAG_RECORD): sgks_backward keeps
                              the adjoint of the basis (d_max x n values, the sweep's largest
                              array, as large as W itself) in pinned host memory mapped into the

@@ -233,6 +233,8 @@ __global__ void __launch_bounds__(kThreads) k_combine(Dims D, Bulk<T> B, Small S
     __shared__ double red[3][kWarps];
     __shared__ int am_last;
     DevScalars* sc = S.sc;
+    // The last CTA of x may set stop while CTAs of e have not started; they then return here and leave part of e as it
+    // was.  Nothing reads e once stop is set (only a new setup clears it, which forms e anew).
     if (sc->stop) return;
     const int d = sc->d, iter = sc->iter;
     for (int j = threadIdx.x; j < D.dmax + kCombCols; j += kThreads) ys[j] = j < d ? (T)S.y[j] : T(0);

@@ -180,8 +180,6 @@ static cudaError_t launch_apply_column(const Dims& D, const DevA<T, V>& A, const
     return cudaGetLastError();
 }
 
-template <typename T> struct GatherAcc { using type = T; };
-
 template <typename T>
 cudaError_t launch_sketch_gather_col(const Dims& D, const Bulk<T>& B, const Small& S, const SketchCSR& SK, cudaStream_t st) {
     carveout_once((const void*)k_sketch_gather_col<T, T, T>);

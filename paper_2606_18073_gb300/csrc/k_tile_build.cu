@@ -352,8 +352,9 @@ struct Build {
     }
 };
 
-// Bit rows of all tiles, with their counts 8 bytes a word: 32 GB at most.  Rays through the whole image
-// with fewer than 2^31 entries stay below it up to 16384^2 pixels; beyond, the row kernels remain.
+// Bit rows of all tiles, with their counts 8 bytes a word: 32 GB at most, for a while.  Rays through the whole image
+// with fewer than 2^31 entries stay below it up to 16384^2 pixels; beyond, and where that memory is not
+// there, the row kernels remain.
 constexpr size_t kMaxWords = (size_t)1 << 32;
 
 // exclusive prefix sums with the total at the end; false when they do not fit
@@ -600,7 +601,9 @@ int build_tiles64(const sgks_reg* reg, const int32_t* rp, const int32_t* ci, con
     Build both(st);   // holds the one layout until the other is there too
     int rc = build_tiles_t(trp, tci, tval, m, n, nnz, reg->nx, reg->ny, nt, tile_ty(B), tile_stage(std::min(B, 8)), t, both.own, st, why);
     if (rc != SGKS_OK || !t.ntiles) return rc;
-    const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, B / kTileInst);   // as measured, also for four instances per CTA
+    // 32 x 16 pixels for the forward pass where the same count of tiles as for the compensated batches allows it: that
+    // pass has up to four times as many CTAs, of four instances, but its tiles are the ones that were measured.
+    const int64_t ctas = (int64_t)((reg->nx + 31) / 32) * ((reg->ny + 15) / 16) * nt * std::max(1, B / kTileInst);
     rc = build_tiles(rp, ci, val, m, n, nnz, reg->nx, reg->ny, nt, ctas < 4 * 152 ? 16 : 32, 16, a, both.own, st, why);
     if (rc != SGKS_OK || !a.ntiles || a.nseg * 4 > nnz) return rc;
     both.keep(allocs);

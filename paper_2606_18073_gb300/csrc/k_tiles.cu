@@ -108,8 +108,8 @@ __device__ __forceinline__ void add_row(Dot2x2 (&acc)[Lanes<IC>::NP], const Stag
 // merge into a sum of full size rounds its low part.  So the terms form a tree, blocks of eight, up to 32 terms of
 // them in a sum of their own, and that into acc: 0.9 to 1.1 times the row kernel's (rms of x after one iteration,
 // float-float, 97^2 with 100, 181^2 with 180 and 256^2 with 30 views).  With 16 instances a stage brings a pixel
-// of a ray operator about 30 terms, so one sum takes them all; HALVES (float-float, fewer instances): the blocks are two
-// chains of four.  512^2 at 64: 2.00 -> 2.18 ms per pass; with fewer instances the same time as before.
+// of a ray operator about 30 terms, so one sum takes them all; HALVES (float-float, fewer instances): each block is
+// two chains of four.  512^2 at 64: 2.00 -> 2.18 ms per pass; with fewer instances the same time as before.
 template <bool HALVES, int IC>
 __device__ __forceinline__ void add_row_tree(Dot2x2 (&acc)[Lanes<IC>::NP], const Staged<float2, IC>& st, Entries& cur,
                                              const uint4* __restrict__ ent, int beg, int end, int next) {
