@@ -17,16 +17,18 @@ def G():
     return G
 
 
-@pytest.mark.parametrize("count,prec", [(2, "ff"), (16, "ff"), (16, "fp32"), (4, "fp64"), (16, "fp64")])
-def test_another_group_changes_no_bits(G, count, prec):
-    A = ct_op(97, np.arange(100) * 1.8, 139)
+# 97^2 is too small for the FP64 tiled passes, 192^2 takes them
+@pytest.mark.parametrize("count,prec,N", [(2, "ff", 97), (16, "ff", 97), (16, "fp32", 97), (4, "fp64", 97),
+                                          (4, "fp64", 192), (16, "fp64", 192)])
+def test_another_group_changes_no_bits(G, count, prec, N):
+    A = ct_op(N, np.arange(40) * 4.5, int(1.43 * N) + 1)
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
     C = G.CSR(dev(A.row_ptr), dev(A.col), dev(A.val.astype(np.float32)), A.m, A.n).transposed()
     g = torch.Generator(device="cuda").manual_seed(2)
     bs = [torch.rand(A.m, generator=g, device="cuda", dtype=torch.float64).to(G.io_dtype(prec)) for _ in range(count + 1)]
     xs = []
     for k in (count, count + 1):   # one group, and the same group with another one beside it
-        Bt = G.Batch([dict(A=C, reg=G.Reg("grad2d", 97, 97), lam=2.0, b=b) for b in bs[:k]], 60, 3, max_iters=5,
+        Bt = G.Batch([dict(A=C, reg=G.Reg("grad2d", N, N), lam=2.0, b=b) for b in bs[:k]], 60, 3, max_iters=5,
                      precision=prec)
         Bt.solve(5)
         xs.append(Bt.x())
